@@ -1203,7 +1203,8 @@ __device__ double closest_on_tri(double3 p, double3 a, double3 b, double3 c, int
     return ddot3(r, r);
 }
 
-__device__ double3 tri_normal64(const Feat &F, int t) {
+// (out of line, as the other rare FP64 paths of k_patch: with few points its time is the fetch of its code)
+__device__ __noinline__ double3 tri_normal64(const Feat &F, int t) {
     double3 a = d3(load_vpos(F.vpos, F.face_vid[3 * t])), b = d3(load_vpos(F.vpos, F.face_vid[3 * t + 1])),
             c = d3(load_vpos(F.vpos, F.face_vid[3 * t + 2]));
     double3 cr = dcross3(b - a, c - a);
@@ -1278,187 +1279,476 @@ __device__ __forceinline__ Cand64 vert_cand64(const Feat &F, double3 p, int v) {
     return c;
 }
 
-// One warp per queued point.  The point's FP32 winner may be wrong by the FP32 error (band edge)
-// or carry an uncertain sign; here the exact FP64 minimum is taken over every feature whose
+// The FP64 re-decision.  A queued point's FP32 winner may be wrong by the FP32 error (band edge) or
+// carry an uncertain sign; here the exact FP64 minimum is taken over every feature whose
 // characteristic region can contain the point: those of the (tile, region) pairs of the point's
 // tile whose tile-local box contains it (every region containing the point is listed there, so
-// the true closest feature is among them, Section 4).  A first FP32 pass over these candidates
+// the true closest feature is among them, Section 4).  An FP32 pass over these candidates
 // finds the smallest FP32 distance d0; only candidates within d0 + 3 delta are evaluated in FP64
 // (the true closest one's FP32 distance is within delta of the minimum, and d0 is at most delta
 // below it, plus the plane distance's under-estimate in the inclusion margin, at most delta).
 // Without a pair list (the paper's cell-loop schedule) the candidates are the triangles of the
 // fans of the FP32 winner's vertices.  The sign is that of (p - q).N with N the FP64 pseudonormal
 // of the feature holding the closest point q (face normal, n1 + n2, or N_alpha, Eq. 8).
+//
+// What bounds it: the latency of the pair and record loads, and the FP64 pipe, which takes some 16
+// cycles per warp instruction whatever the number of active lanes.  So each phase of a round (up to
+// 32 points per block) fills its lanes:
+//   0. one thread per point finds the point's tile and pairs;
+//   1. a warp per point reads the tile's pairs, the next four loads in flight, and queues those whose box
+//      holds the point; the distances of 32 queued regions are evaluated at once (a box test per
+//      lane with the distance behind it left most lanes idle).  A tile of more than PB_SHARE pairs
+//      is shared by the block's warps, so that the largest tile does not set the kernel's time;
+//   2. the FP64 candidates of all points (about 1.5 each) are spread over the block's threads,
+//      one each, instead of a warp per point;
+//   3. one thread per point takes the sign and writes the result.
+// With a warp per point throughout, the kernel took 184 us on the 2.1 M-triangle knot at 512^3
+// (2,085 points, about 1,200 pairs per tile), 264 us at 1024^3 (16,855 points) and 40 us on the
+// 50 k-triangle torus at 512^3 (1,657 points); now 46, 93 and 17 us.
+constexpr int PB_WARPS = 4;              // warps per block
+constexpr int PATCH_NT = 32 * PB_WARPS;
+constexpr int PB_PTS = 4 * PB_WARPS;     // points of a round
+constexpr int PB_QUEUE = 128;            // FP64 candidates of a round
+constexpr int PB_LIST = 64;              // FP32 survivors a warp keeps for its point
+// Pairs of a tile that one warp reads alone.  Sharing a tile costs every warp the start of its part
+// (about 2 us): from 512 pairs on it took the knot at 1024^3 (436 pairs per tile) from 109 to 167 us;
+// never sharing, the batch of 24 uneven meshes (tiles of up to 10^4 pairs) took 85 instead of 36 us.
+constexpr int PB_SHARE = 2048;
+
+struct PatchSmem {
+    int hit[PB_WARPS][256];              // regions whose box holds the warp's point (a ring)
+    int cand_fid[PB_WARPS][PB_LIST];     // those within the FP32 threshold, and their distances
+    float cand_d[PB_WARPS][PB_LIST];
+    // the round's FP64 candidates: entries [0, PB_QUEUE) hold regions to evaluate, entry
+    // PB_QUEUE + PB_WARPS t + w what warp w evaluated itself for point t (more than the queue has room for)
+    int q_fid[PB_QUEUE];
+    float q_d[PB_QUEUE];
+    int q_pt[PB_QUEUE + PB_PTS * PB_WARPS];  // their points, -1: none
+    double r_d2[PB_QUEUE + PB_PTS * PB_WARPS];
+    int r_id[PB_QUEUE + PB_PTS * PB_WARPS];
+    double r_pq[PB_QUEUE + PB_PTS * PB_WARPS][3];
+    int nq;
+    // per point of the round
+    int4 ijk[PB_PTS];                    // grid indices, problem
+    long long idx[PB_PTS];
+    long long q0[PB_PTS];                // its tile's pairs, and its place in the tile
+    int nq_pairs[PB_PTS], local[PB_PTS];
+    int fid[PB_PTS];                     // the FP32 winner
+    unsigned d0[PB_PTS];                 // smallest FP32 distance (the bits of a float >= 0 order like it)
+    unsigned long long d2[PB_PTS];       // smallest FP64 squared distance, likewise
+    int id[PB_PTS];                      // the closest feature, the smallest id at equal distance
+    int src[PB_PTS];                     // the entry that holds it
+};
+
+__device__ __forceinline__ double3 grid_point64(const GridP &g, int i, int j, int k) {
+    const double h = g.h;
+    return make_double3((double)g.ox + (i + 0.5) * h, (double)g.oy + (j + 0.5) * h,
+                        (double)g.oz + (k + g.kofs + 0.5) * h);
+}
+
+__device__ __forceinline__ Cand64 feature_cand64(const Feat &F, double3 p, int fid) {
+    const int type = feat_type(F, fid), id = feat_local(F, fid, type);
+    return type == FACE ? face_cand64(F, p, id) : (type == EDGE ? edge_cand64(F, p, id) : vert_cand64(F, p, id));
+}
+
+// The smallest candidate of the warp's lanes, as the entry of this warp for point t.
+__device__ __forceinline__ void warp_result64(PatchSmem &S, int t, Cand64 best) {
+    int src = (int)(threadIdx.x & 31);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double od = __shfl_xor_sync(FULL, best.d2, off);
+        const int oid = __shfl_xor_sync(FULL, best.id, off);
+        const int os = __shfl_xor_sync(FULL, src, off);
+        if (cand_less(od, oid, best.d2, best.id)) { best.d2 = od; best.id = oid; src = os; }
+    }
+    const double3 pq = make_double3(__shfl_sync(FULL, best.pq.x, src), __shfl_sync(FULL, best.pq.y, src),
+                                    __shfl_sync(FULL, best.pq.z, src));
+    if ((threadIdx.x & 31) == 0) {
+        const int e = PB_QUEUE + t * PB_WARPS + (int)(threadIdx.x >> 5);
+        S.r_d2[e] = best.d2;
+        S.r_id[e] = best.id;
+        S.r_pq[e][0] = pq.x;
+        S.r_pq[e][1] = pq.y;
+        S.r_pq[e][2] = pq.z;
+        S.q_pt[e] = t;
+    }
+}
+
+// FP64 candidates of a warp's list of m features, in place of the block's queue: for a point with
+// more of them than fit (a vertex fan of hundreds of faces at one distance).
+__device__ __noinline__ void list_cand64(const Feat &F, const GridP &g, int4 ijk, const int *fids, int m,
+                                         Cand64 &best) {
+    const double3 p = grid_point64(g, ijk.x, ijk.y, ijk.z);
+    for (int e = (int)(threadIdx.x & 31); e < m; e += 32) {
+        const Cand64 c = feature_cand64(F, p, fids[e]);
+        if (cand_less(c.d2, c.id, best.d2, best.id)) best = c;
+    }
+}
+
+// Phase 0 for point t of the round, by one thread.
 template <int TY, int TZ>
-__global__ void __launch_bounds__(256) k_patch(const Prob *P, const long long *tile_base, Outputs o) {
+__device__ __forceinline__ void patch_locate(const Prob *P, const long long *tile_base, const Outputs &o, PatchEntry pe,
+                                             int t, PatchSmem &S) {
+    const GridP &g = P[pe.prob].g;
+    const int64_t idx = pe.idx, plane = (int64_t)g.nx * g.ny;
+    int gi, gj, gk;
+    if (idx < (int64_t(1) << 31)) {
+        const uint32_t iu = (uint32_t)idx, r1 = g.div_nx.div(iu), r2 = g.div_ny.div(r1);
+        gi = (int)(iu - r1 * (uint32_t)g.nx);
+        gj = (int)(r1 - r2 * (uint32_t)g.ny);
+        gk = (int)r2;
+    } else {
+        gk = (int)(idx / plane);
+        gj = (int)((idx - (int64_t)gk * plane) / g.nx);
+        gi = (int)(idx - (int64_t)gk * plane - (int64_t)gj * g.nx);
+    }
+    S.ijk[t] = make_int4(gi, gj, gk, pe.prob);
+    S.idx[t] = idx;
+    S.d0[t] = 0x7f800000u;            // +inf
+    S.d2[t] = 0x7ff0000000000000ull;  // +inf
+    S.id[t] = 0x7fffffff;
+    S.src[t] = 0x7fffffff;
+    if (o.pairs) {
+        const int tx = gi / TILE_X, ty = gj / TY, tz = gk / TZ;
+        const int64_t tile = tile_base[pe.prob] + ((int64_t)tz * g.nty + ty) * g.ntx + tx;
+        const uint32_t *st = o.bin_start + 3 * tile;
+        const int64_t q0 = min((int64_t)st[0], o.pair_cap), q3 = min((int64_t)st[3], o.pair_cap);
+        S.q0[t] = q0;
+        S.nq_pairs[t] = (int)(q3 - q0);
+        S.local[t] = (gi - tx * TILE_X) | (gj - ty * TY) << 8 | (gk - tz * TZ) << 16;
+        S.fid[t] = pe.fid;
+    } else {  // no pair list: the FP32 winner
+        S.q0[t] = 0;
+        S.nq_pairs[t] = 0;
+        S.fid[t] = pe.fid;
+    }
+}
+
+// Phase 1 without a pair list: the fans of the FP32 winner's vertices, concatenated; lanes take one
+// corner (triangle) each.
+__device__ __noinline__ void patch_fans(const Feat &F, const GridP &g, int t, PatchSmem &S) {
+    const int lane = threadIdx.x & 31;
+    const int4 ijk = S.ijk[t];
+    const double3 p = grid_point64(g, ijk.x, ijk.y, ijk.z);
+    Cand64 best;
+    best.d2 = INFINITY;
+    best.id = 0x7fffffff;
+    best.pq = make_double3(0, 0, 0);
+    const int fid = S.fid[t];
+    int vs[3], nv;
+    if (fid < F.T) { vs[0] = F.face_vid[3 * fid]; vs[1] = F.face_vid[3 * fid + 1]; vs[2] = F.face_vid[3 * fid + 2]; nv = 3; }
+    else if (fid < F.T + F.E) { int4 q = F.edge_vf[fid - F.T]; vs[0] = q.x; vs[1] = q.y; vs[2] = 0; nv = 2; }
+    else { vs[0] = fid - F.T - F.E; vs[1] = vs[2] = 0; nv = 1; }
+    int c0[3], cn[3];
+    for (int a = 0; a < 3; a++) {
+        c0[a] = a < nv ? F.vert_start[vs[a]] : 0;
+        cn[a] = a < nv ? F.vert_start[vs[a] + 1] - c0[a] : 0;
+    }
+    const int total = cn[0] + cn[1] + cn[2];
+    for (int slot = lane; slot < total; slot += 32) {
+        const int a = slot < cn[0] ? 0 : (slot < cn[0] + cn[1] ? 1 : 2);
+        const int c = c0[a] + slot - (a == 0 ? 0 : (a == 1 ? cn[0] : cn[0] + cn[1]));
+        const Cand64 cd = face_cand64(F, p, F.vert_corner[c] / 3);
+        if (cand_less(cd.d2, cd.id, best.d2, best.id)) best = cd;
+    }
+    __syncwarp();
+    warp_result64(S, t, best);
+}
+
+// eval_any's distance where it may be at most `lim`, +inf where it is surely larger: most of the
+// faces whose box holds the point hold it outside their prism, and there the distances to the face's
+// plane and past its side planes (each within delta of their true values, like the distance itself)
+// spare the three segments of the triangle's boundary.
+__device__ __forceinline__ float eval_within(const Feat &F, const GridP &g, int fid, int4 ijk, float lim) {
+    const int type = feat_type(F, fid), id = feat_local(F, fid, type);
+    if (type == FACE) {
+        const float3 p = make_float3(fmaf((float)ijk.x + 0.5f, g.h, g.ox), fmaf((float)ijk.y + 0.5f, g.h, g.oy),
+                                     fmaf((float)(ijk.z + g.kofs) + 0.5f, g.h, g.oz));
+        const float4 *r = F.face_rec + 4 * id;
+        const float4 n = __ldg(r), s1 = __ldg(r + 1), s2 = __ldg(r + 2), s3 = __ldg(r + 3);
+        const float sd = fabsf(dot3(f3(n), p) + n.w);
+        const float out = -fminf(fminf(dot3(f3(s1), p) + s1.w, dot3(f3(s2), p) + s2.w), dot3(f3(s3), p) + s3.w);
+        if (fmaxf(sd, out) > lim + 2.f * g.derr) return INFINITY;
+    }
+    bool neg, unc;
+    return eval_any(F, g, type, id, ijk.x, ijk.y, ijk.z, neg, unc);
+}
+
+// Phase 1 for point t of the round and n of its tile's pairs from q0 on, by one warp.
+__device__ __forceinline__ void patch_scan(const Prob *P, const Outputs &o, int64_t q0, int n, int t, PatchSmem &S) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int4 ijk = S.ijk[t];
+    const Feat &F = P[ijk.w].F;
+    const GridP &g = P[ijk.w].g;
+    const int64_t q3 = q0 + n;
+    const unsigned lx = (unsigned)S.local[t] & 255u, ly = ((unsigned)S.local[t] >> 8) & 255u,
+                   lz = (unsigned)S.local[t] >> 16;
+    Cand64 best;  // (used by list_cand64 only)
+    best.d2 = INFINITY;
+    best.id = 0x7fffffff;
+    best.pq = make_double3(0, 0, 0);
+    const unsigned lt_mask = (1u << lane) - 1u;
+    int *const hit = S.hit[warp], *const lf = S.cand_fid[warp];
+    float *const ld = S.cand_d[warp];
+    const float slack = 3.f * g.derr;
+    float d0 = __uint_as_float(S.d0[t]);
+    int h0 = 0, nh = 0, nc = 0;  // ring start and length, survivors (warp-uniform)
+    bool direct = false;         // survivors were already evaluated in FP64 (best)
+    // drops the survivors that the smaller d0 rules out
+    auto tighten = [&]() {
+        const float thr = d0 + slack;
+        int m = 0;
+        for (int e0 = 0; e0 < nc; e0 += 32) {
+            const int e = e0 + lane;
+            const int f = e < nc ? lf[e] : 0;
+            const float d = e < nc ? ld[e] : INFINITY;
+            const bool keep = e < nc && d <= thr;
+            const unsigned km = __ballot_sync(FULL, keep);  // (and every read above precedes the writes)
+            if (keep) {
+                lf[m + __popc(km & lt_mask)] = f;
+                ld[m + __popc(km & lt_mask)] = d;
+            }
+            m += __popc(km);
+            __syncwarp();
+        }
+        nc = m;
+    };
+    // FP32 distances of n <= 32 queued regions
+    auto evaluate = [&](int n) {
+        const int fid = lane < n ? hit[(h0 + lane) & 255] : 0;
+        const float d = lane < n ? eval_within(F, g, fid, ijk, d0 + slack) : INFINITY;
+        float m = d;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fminf(m, __shfl_xor_sync(FULL, m, off));
+        d0 = fminf(d0, m);
+        const bool keep = d <= d0 + slack && lane < n;
+        const unsigned km = __ballot_sync(FULL, keep);
+        if (nc + __popc(km) > PB_LIST) {
+            tighten();
+            if (nc + __popc(km) > PB_LIST) {
+                list_cand64(F, g, ijk, lf, nc, best);
+                __syncwarp();
+                nc = 0;
+                direct = true;
+            }
+        }
+        if (keep) {
+            lf[nc + __popc(km & lt_mask)] = fid;
+            ld[nc + __popc(km & lt_mask)] = d;
+        }
+        nc += __popc(km);
+        h0 = (h0 + n) & 255;
+        nh -= n;
+        __syncwarp();
+    };
+    int2 pr[4], next[4];
+    auto load = [&](int64_t q, int2 *v) {
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int64_t qq = q + 32 * u + lane;
+            v[u] = qq < q3 ? __ldg(o.pairs + qq) : make_int2(0, 31);  // (a box that is empty along x)
+        }
+    };
+    load(q0, next);
+    {   // the winner is one of the tile's regions: its distance bounds the smallest one
+        const int type = feat_type(F, S.fid[t]);
+        bool neg, unc;
+        d0 = fminf(d0, eval_any(F, g, type, feat_local(F, S.fid[t], type), ijk.x, ijk.y, ijk.z, neg, unc));
+    }
+    for (int64_t q = q0; q < q3; q += 128) {
+#pragma unroll
+        for (int u = 0; u < 4; u++) pr[u] = next[u];
+        load(q + 128, next);  // in flight while this step's regions are tested and evaluated
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const unsigned bx = (unsigned)pr[u].y;
+            const bool in = lx >= (bx & 31u) && lx <= ((bx >> 5) & 31u) && ly >= ((bx >> 10) & 15u) &&
+                            ly <= ((bx >> 14) & 15u) && lz >= ((bx >> 18) & 15u) && lz <= ((bx >> 22) & 15u);
+            const unsigned hm = __ballot_sync(FULL, in);
+            if (in) hit[(h0 + nh + __popc(hm & lt_mask)) & 255] = pr[u].x;
+            nh += __popc(hm);
+        }
+        __syncwarp();
+        while (nh >= 32) evaluate(32);
+    }
+    if (nh > 0) evaluate(nh);
+    tighten();
+    if (lane == 0) atomicMin(&S.d0[t], __float_as_uint(d0));
+    int at = 0;
+    if (lane == 0 && !direct && nc > 0) at = atomicAdd(&S.nq, nc);
+    at = __shfl_sync(FULL, at, 0);
+    if (direct || at + nc > PB_QUEUE) {
+        list_cand64(F, g, ijk, lf, nc, best);
+        __syncwarp();
+        warp_result64(S, t, best);
+    } else {
+        for (int e = lane; e < nc; e += 32) {
+            S.q_fid[at + e] = lf[e];
+            S.q_d[at + e] = ld[e];
+            S.q_pt[at + e] = t;
+        }
+    }
+    __syncwarp();
+}
+
+// FP64 pseudonormal of vertex u (Eq. 8) by one warp, N_alpha = sum alpha_i n_i, lanes over the fan
+__device__ __noinline__ double3 fan_normal64(const Feat &F, int u) {
+    const int lane = threadIdx.x & 31;
+    const int c0 = F.vert_start[u], c1 = F.vert_start[u + 1];
+    const double3 Pv = d3(load_vpos(F.vpos, u));
+    double3 acc = make_double3(0, 0, 0);
+    for (int c = c0 + lane; c < c1; c += 32) {
+        const int cc = F.vert_corner[c];
+        const int ft = cc / 3, kk = cc - 3 * ft;
+        double3 e1 = d3(load_vpos(F.vpos, F.face_vid[3 * ft + (kk + 1) % 3])) - Pv;
+        double3 e2 = d3(load_vpos(F.vpos, F.face_vid[3 * ft + (kk + 2) % 3])) - Pv;
+        double3 cr = dcross3(e1, e2);
+        double alpha = atan2(sqrt(ddot3(cr, cr)), ddot3(e1, e2));
+        acc = acc + alpha * tri_normal64(F, ft);
+    }
+    return make_double3(wsum(acc.x), wsum(acc.y), wsum(acc.z));
+}
+
+// Phase 3 for one point of the round per lane (has: the lane has one), by one warp.
+__device__ __forceinline__ void patch_write(const Prob *P, const Outputs &o, const PatchSmem &S, int t, bool has) {
+    const int lane = threadIdx.x & 31;
+    const int prob = has ? S.ijk[t].w : 0;
+    const Feat &F = P[prob].F;
+    const int out_id = has ? S.id[t] : 0x7fffffff;
+    const double best_d2 = has ? __longlong_as_double((long long)S.d2[t]) : INFINITY;
+    const int src = has ? S.src[t] : 0x7fffffff;
+    const double3 pq = src != 0x7fffffff ? make_double3(S.r_pq[src][0], S.r_pq[src][1], S.r_pq[src][2])
+                                         : make_double3(0, 0, 0);
+    // The sign: (p - q).N with the feature's stored FP32 pseudonormal (face normal, n1 + n2, unit
+    // N_alpha) when that cannot flip it, i.e. when |(p - q).N| exceeds |p - q| times the stored
+    // normal's direction error (u for faces and edges, rounded from FP64 normals; tau_v for
+    // N_alpha); otherwise the FP64 pseudonormal (Eq. 8 for a vertex).  The fallback is rare: it
+    // needs p within about 1e-6 |p - q| of the pseudonormal's plane.
+    const double pq2 = ddot3(pq, pq);
+    double3 N = make_double3(0, 0, 0);
+    double nerr = 0.0;
+    if (out_id == 0x7fffffff) {
+        // no candidate (or no point in this lane)
+    } else if (out_id < F.T) {
+        N = d3(f3(__ldg(F.face_rec + 4 * out_id)));
+        nerr = 4e-7;
+    } else if (out_id < F.T + F.E) {
+        N = d3(f3(__ldg(F.edge_rec + 5 * (out_id - F.T) + 4)));
+        nerr = 8e-7;
+    } else {
+        N = d3(f3(__ldg(F.vert_rec + 3 * (out_id - F.T - F.E) + 1)));
+        nerr = (double)__uint_as_float(F.prec[PREC_TAU_V]) + 4e-7;
+    }
+    // |(p - q).N| > 2 nerr |p - q| |N|, squared (no FP64 square roots: they are long sequences
+    // on this part's FP64 pipe)
+    const double sN = ddot3(pq, N);
+    const bool sure = out_id == 0x7fffffff || sN * sN > 4.0 * nerr * nerr * pq2 * ddot3(N, N) + 1e-300;
+    bool fan = false;  // the vertex's FP64 pseudonormal is wanted
+    if (sure) {
+        // the stored normal decides
+    } else if (out_id < F.T) {
+        N = tri_normal64(F, out_id);
+    } else if (out_id < F.T + F.E) {
+        const int4 q = F.edge_vf[out_id - F.T];
+        N = tri_normal64(F, q.z) + tri_normal64(F, q.w);
+    } else {
+        fan = true;
+    }
+    for (unsigned todo = __ballot_sync(FULL, fan); todo; todo &= todo - 1) {
+        const int who = __ffs(todo) - 1;
+        const Feat &G = P[__shfl_sync(FULL, prob, who)].F;
+        const int u = __shfl_sync(FULL, out_id, who) - G.T - G.E;
+        const double3 acc = fan_normal64(G, u);
+        if (lane == who) N = acc;
+    }
+    if (!has) return;
+    const Prob &pr = P[prob];
+    const double s = ddot3(pq, N);
+    float val = INFINITY;
+    int w = -1;
+    // |d| < w decided on the squares (w^2 is exact in FP64); the value is the FP32 square root
+    // of the FP64 square distance (within an FP32 ulp of the rounded FP64 distance)
+    if (best_d2 < (double)pr.g.w * (double)pr.g.w) {
+        const float d = sqrtf((float)best_d2);
+        val = s < 0.0 ? -d : d;
+        w = out_id;
+    }
+    const int64_t idx = S.idx[t];
+    if (pr.dist) pr.dist[idx] = val;
+    if (pr.winner) pr.winner[idx] = w;
+    if (pr.list && w >= 0) {
+        const unsigned long long pos = atomicAdd(pr.list_count, 1ull);
+        if ((long long)pos < pr.list_cap) {
+            pr.list[pos] = make_uint2((uint32_t)idx, (uint32_t)w);
+            if (pr.list_dist) pr.list_dist[pos] = val;
+        } else {
+            atomicOr(&o.ctr->nb_status, ST_LIST_OVERFLOW);
+        }
+    }
+}
+
+template <int TY, int TZ>
+__global__ void __launch_bounds__(PATCH_NT, 4) k_patch(const Prob *P, const long long *tile_base, Outputs o) {
     dep_wait();
     dep_next();
-    const int lane = threadIdx.x & 31;
-    const int64_t wid0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    __shared__ PatchSmem S;
+    const int warp = threadIdx.x >> 5;
     const int64_t n = min((int64_t)o.ctr->n_patch, o.patch_cap);
-    for (int64_t e = wid0; e < n; e += nwarps) {
-        PatchEntry pe = o.patch[e];
-        const int64_t idx = pe.idx;
-        const int fid = pe.fid;
-        const Feat &F = P[pe.prob].F;
-        const GridP &g = P[pe.prob].g;
-        float *const dist = P[pe.prob].dist;
-        int32_t *const winner = P[pe.prob].winner;
-        const int64_t plane = (int64_t)g.nx * g.ny;
-        int gi, gj, gk;
-        if (idx < (int64_t(1) << 31)) {
-            const uint32_t iu = (uint32_t)idx, r1 = g.div_nx.div(iu), r2 = g.div_ny.div(r1);
-            gi = (int)(iu - r1 * (uint32_t)g.nx);
-            gj = (int)(r1 - r2 * (uint32_t)g.ny);
-            gk = (int)r2;
-        } else {
-            gk = (int)(idx / plane);
-            gj = (int)((idx - (int64_t)gk * plane) / g.nx);
-            gi = (int)(idx - (int64_t)gk * plane - (int64_t)gj * g.nx);
+    // points per warp and round: a few thousand points take one round over all blocks
+    const int64_t warps = (int64_t)gridDim.x * PB_WARPS;
+    const int round = n <= warps ? PB_WARPS : (n <= 2 * warps ? 2 * PB_WARPS : PB_PTS);
+    for (int64_t e0 = (int64_t)blockIdx.x * round; e0 < n; e0 += (int64_t)gridDim.x * round) {
+        const int np = (int)min((int64_t)round, n - e0);
+        if (threadIdx.x == 0) S.nq = 0;
+        for (int e = threadIdx.x; e < PB_QUEUE + PB_PTS * PB_WARPS; e += PATCH_NT) S.q_pt[e] = -1;
+        if ((int)threadIdx.x < np) patch_locate<TY, TZ>(P, tile_base, o, o.patch[e0 + threadIdx.x], threadIdx.x, S);
+        __syncthreads();
+        for (int t = 0; t < np; t++) {
+            const int m = S.nq_pairs[t];
+            if (m <= PB_SHARE) {  // this warp's own points
+                if (t % PB_WARPS != warp) continue;
+                if (!o.pairs) patch_fans(P[S.ijk[t].w].F, P[S.ijk[t].w].g, t, S);
+                else if (m > 0) patch_scan(P, o, S.q0[t], m, t, S);
+            } else {  // its share of the tile's pairs
+                const int a = (int)((int64_t)m * warp / PB_WARPS), b = (int)((int64_t)m * (warp + 1) / PB_WARPS);
+                patch_scan(P, o, S.q0[t] + a, b - a, t, S);
+            }
         }
-        const double h = g.h;
-        const double3 p = make_double3((double)g.ox + (gi + 0.5) * h, (double)g.oy + (gj + 0.5) * h,
-                                       (double)g.oz + (gk + g.kofs + 0.5) * h);
-        Cand64 best;
-        best.d2 = INFINITY;
-        best.id = 0x7fffffff;
-        best.pq = make_double3(0, 0, 0);
-        if (o.pairs) {
-            const int tx = gi / TILE_X, ty = gj / TY, tz = gk / TZ;
-            const int64_t tile = tile_base[pe.prob] + ((int64_t)tz * g.nty + ty) * g.ntx + tx;
-            const uint32_t *st = o.bin_start + 3 * tile;
-            const int64_t q0 = min((int64_t)st[0], o.pair_cap), q3 = min((int64_t)st[3], o.pair_cap);
-            const unsigned lx = (unsigned)(gi - tx * TILE_X), ly = (unsigned)(gj - ty * TY), lz = (unsigned)(gk - tz * TZ);
-            // pass 1: the smallest FP32 distance over the regions whose box holds the point
-            float d0 = INFINITY;
-            for (int64_t q = q0 + lane; q < q3; q += 32) {
-                const int2 pr = __ldg(o.pairs + q);
-                const unsigned bx = (unsigned)pr.y;
-                if (lx < (bx & 31u) || lx > ((bx >> 5) & 31u) || ly < ((bx >> 10) & 15u) || ly > ((bx >> 14) & 15u) ||
-                    lz < ((bx >> 18) & 15u) || lz > ((bx >> 22) & 15u))
+        __syncthreads();
+        // phase 2: the FP64 candidates; per point the smallest (distance, feature id)
+        for (int e = threadIdx.x; e < PB_QUEUE + PB_PTS * PB_WARPS; e += PATCH_NT) {
+            const int t = S.q_pt[e];
+            if (t < 0) continue;
+            if (e < PB_QUEUE) {
+                const int4 ijk = S.ijk[t];
+                const Prob &pr = P[ijk.w];
+                if (!(S.q_d[e] <= __uint_as_float(S.d0[t]) + 3.f * pr.g.derr)) {  // another warp found a closer region
+                    S.q_pt[e] = -1;
                     continue;
-                const int type = feat_type(F, pr.x);
-                bool neg, unc;
-                d0 = fminf(d0, eval_any(F, g, type, feat_local(F, pr.x, type), gi, gj, gk, neg, unc));
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) d0 = fminf(d0, __shfl_xor_sync(FULL, d0, off));
-            const float thr = d0 + 3.f * g.derr;
-            // pass 2: FP64 closest points of the candidates within the threshold
-            for (int64_t q = q0 + lane; q < q3; q += 32) {
-                const int2 pr = __ldg(o.pairs + q);
-                const unsigned bx = (unsigned)pr.y;
-                if (lx < (bx & 31u) || lx > ((bx >> 5) & 31u) || ly < ((bx >> 10) & 15u) || ly > ((bx >> 14) & 15u) ||
-                    lz < ((bx >> 18) & 15u) || lz > ((bx >> 22) & 15u))
-                    continue;
-                const int type = feat_type(F, pr.x), id = feat_local(F, pr.x, type);
-                bool neg, unc;
-                if (!(eval_any(F, g, type, id, gi, gj, gk, neg, unc) <= thr)) continue;
-                const Cand64 c = type == FACE ? face_cand64(F, p, id) : (type == EDGE ? edge_cand64(F, p, id)
-                                                                                       : vert_cand64(F, p, id));
-                if (cand_less(c.d2, c.id, best.d2, best.id)) best = c;
-            }
-        } else {
-            // the fans of the winner's vertices, concatenated; lanes take one corner (triangle) each
-            int vs[3], nv;
-            if (fid < F.T) { vs[0] = F.face_vid[3 * fid]; vs[1] = F.face_vid[3 * fid + 1]; vs[2] = F.face_vid[3 * fid + 2]; nv = 3; }
-            else if (fid < F.T + F.E) { int4 q = F.edge_vf[fid - F.T]; vs[0] = q.x; vs[1] = q.y; vs[2] = 0; nv = 2; }
-            else { vs[0] = fid - F.T - F.E; vs[1] = vs[2] = 0; nv = 1; }
-            int c0[3], cn[3];
-            for (int a = 0; a < 3; a++) {
-                c0[a] = a < nv ? F.vert_start[vs[a]] : 0;
-                cn[a] = a < nv ? F.vert_start[vs[a] + 1] - c0[a] : 0;
-            }
-            const int total = cn[0] + cn[1] + cn[2];
-            for (int slot = lane; slot < total; slot += 32) {
-                const int a = slot < cn[0] ? 0 : (slot < cn[0] + cn[1] ? 1 : 2);
-                const int c = c0[a] + slot - (a == 0 ? 0 : (a == 1 ? cn[0] : cn[0] + cn[1]));
-                const Cand64 cd = face_cand64(F, p, F.vert_corner[c] / 3);
-                if (cand_less(cd.d2, cd.id, best.d2, best.id)) best = cd;
-            }
-        }
-        // warp argmin over (d2, feature id)
-        int src = lane;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double od = __shfl_xor_sync(FULL, best.d2, off);
-            const int oid = __shfl_xor_sync(FULL, best.id, off);
-            const int os = __shfl_xor_sync(FULL, src, off);
-            if (cand_less(od, oid, best.d2, best.id)) { best.d2 = od; best.id = oid; src = os; }
-        }
-        const double3 pq = make_double3(__shfl_sync(FULL, best.pq.x, src), __shfl_sync(FULL, best.pq.y, src),
-                                        __shfl_sync(FULL, best.pq.z, src));
-        const int out_id = best.id;
-        // The sign: (p - q).N with the feature's stored FP32 pseudonormal (face normal, n1 + n2, unit
-        // N_alpha) when that cannot flip it, i.e. when |(p - q).N| exceeds |p - q| times the stored
-        // normal's direction error (u for faces and edges, rounded from FP64 normals; tau_v for
-        // N_alpha); otherwise the FP64 pseudonormal (Eq. 8 for a vertex).  The fallback is rare: it
-        // needs p within about 1e-6 |p - q| of the pseudonormal's plane.
-        const double pq2 = ddot3(pq, pq);
-        double3 N = make_double3(0, 0, 0);
-        double nerr = 0.0;
-        if (out_id < F.T) {
-            N = d3(f3(__ldg(F.face_rec + 4 * out_id)));
-            nerr = 4e-7;
-        } else if (out_id < F.T + F.E) {
-            N = d3(f3(__ldg(F.edge_rec + 5 * (out_id - F.T) + 4)));
-            nerr = 8e-7;
-        } else if (out_id != 0x7fffffff) {
-            N = d3(f3(__ldg(F.vert_rec + 3 * (out_id - F.T - F.E) + 1)));
-            nerr = (double)__uint_as_float(F.prec[PREC_TAU_V]) + 4e-7;
-        }
-        // |(p - q).N| > 2 nerr |p - q| |N|, squared (no FP64 square roots: they are long sequences
-        // on this part's FP64 pipe, which bounds this kernel)
-        const double sN = ddot3(pq, N);
-        const bool sure = sN * sN > 4.0 * nerr * nerr * pq2 * ddot3(N, N) + 1e-300;
-        if (sure) {
-            // the stored normal decides
-        } else if (out_id < F.T) {
-            N = tri_normal64(F, out_id);
-        } else if (out_id < F.T + F.E) {
-            const int4 q = F.edge_vf[out_id - F.T];
-            N = tri_normal64(F, q.z) + tri_normal64(F, q.w);
-        } else if (out_id != 0x7fffffff) {
-            const int u = out_id - F.T - F.E;
-            const int c0 = F.vert_start[u], c1 = F.vert_start[u + 1];
-            const double3 Pv = d3(load_vpos(F.vpos, u));
-            double3 acc = make_double3(0, 0, 0);
-            for (int c = c0 + lane; c < c1; c += 32) {  // N_alpha = sum alpha_i n_i, lanes over the fan
-                const int cc = F.vert_corner[c];
-                const int ft = cc / 3, kk = cc - 3 * ft;
-                double3 e1 = d3(load_vpos(F.vpos, F.face_vid[3 * ft + (kk + 1) % 3])) - Pv;
-                double3 e2 = d3(load_vpos(F.vpos, F.face_vid[3 * ft + (kk + 2) % 3])) - Pv;
-                double3 cr = dcross3(e1, e2);
-                double alpha = atan2(sqrt(ddot3(cr, cr)), ddot3(e1, e2));
-                acc = acc + alpha * tri_normal64(F, ft);
-            }
-            N = make_double3(wsum(acc.x), wsum(acc.y), wsum(acc.z));
-        }
-        const double s = ddot3(pq, N);
-        if (lane == 0) {
-            float val = INFINITY;
-            int w = -1;
-            // |d| < w decided on the squares (w^2 is exact in FP64); the value is the FP32 square root
-            // of the FP64 square distance (within an FP32 ulp of the rounded FP64 distance)
-            if (best.d2 < (double)g.w * (double)g.w) {
-                const float d = sqrtf((float)best.d2);
-                val = s < 0.0 ? -d : d;
-                w = out_id;
-            }
-            if (dist) dist[idx] = val;
-            if (winner) winner[idx] = w;
-            const Prob &pr = P[pe.prob];
-            if (pr.list && w >= 0) {
-                const unsigned long long pos = atomicAdd(pr.list_count, 1ull);
-                if ((long long)pos < pr.list_cap) {
-                    pr.list[pos] = make_uint2((uint32_t)idx, (uint32_t)w);
-                    if (pr.list_dist) pr.list_dist[pos] = val;
-                } else {
-                    atomicOr(&o.ctr->nb_status, ST_LIST_OVERFLOW);
                 }
+                const Cand64 c = feature_cand64(pr.F, grid_point64(pr.g, ijk.x, ijk.y, ijk.z), S.q_fid[e]);
+                S.r_d2[e] = c.d2;
+                S.r_id[e] = c.id;
+                S.r_pq[e][0] = c.pq.x;
+                S.r_pq[e][1] = c.pq.y;
+                S.r_pq[e][2] = c.pq.z;
             }
+            atomicMin(&S.d2[t], (unsigned long long)__double_as_longlong(S.r_d2[e]));  // d2 >= 0
         }
+        __syncthreads();
+        for (int e = threadIdx.x; e < PB_QUEUE + PB_PTS * PB_WARPS; e += PATCH_NT) {
+            const int t = S.q_pt[e];
+            if (t >= 0 && (unsigned long long)__double_as_longlong(S.r_d2[e]) == S.d2[t]) atomicMin(&S.id[t], S.r_id[e]);
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < PB_QUEUE + PB_PTS * PB_WARPS; e += PATCH_NT) {
+            const int t = S.q_pt[e];
+            if (t >= 0 && (unsigned long long)__double_as_longlong(S.r_d2[e]) == S.d2[t] && S.r_id[e] == S.id[t])
+                atomicMin(&S.src[t], e);
+        }
+        __syncthreads();
+        if (warp == 0) patch_write(P, o, S, (int)threadIdx.x, (int)threadIdx.x < np);
+        __syncthreads();
     }
 }
 
@@ -1746,7 +2036,7 @@ template <int TY, int TZ, bool LIST, bool SPLIT = false> static int tile_blocks_
 template <int TY, int TZ> static int patch_blocks() {
     static int b = 0;
     if (!b) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_patch<TY, TZ>, 256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_patch<TY, TZ>, PATCH_NT, 0);
         if (b <= 0) b = 1;
         b *= num_sms();
     }
@@ -2224,7 +2514,7 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
                            (const int32_t *)sc.empty_list, sc.band_pos + n_tiles, sc.ticket, sc.any_dense ? 1 : 0));
     }
     if (ev) SDF_TRY(record_event(ev[2], s));
-    SDF_TRY(launch_dep(k_patch<TY, TZ>, dim3(patch_blocks<TY, TZ>()), dim3(256), 0, s, sc.probs, sc.tbase, o));
+    SDF_TRY(launch_dep(k_patch<TY, TZ>, dim3(patch_blocks<TY, TZ>()), dim3(PATCH_NT), 0, s, sc.probs, sc.tbase, o));
     if (sc.fprobs)
         SDF_TRY(fill_sign(sc.fprobs, sc.rbase, sc.zbase, sc.ybase, n, sc.r_tot, sc.z_tot, sc.y_tot, sc.rowsign,
                           num_sms(), s));
@@ -2255,7 +2545,7 @@ static int launch_cell_loop(int n, long long f_tot, const Scratch &sc, cudaStrea
     SDF_LAUNCHED(1);
     SDF_TRY(cudaGetLastError());
     if (ev) SDF_TRY(record_event(ev[2], s));
-    k_patch<8, 8><<<patch_blocks<8, 8>(), 256, 0, s>>>(sc.probs, sc.tbase, o);  // no pairs: fan search
+    k_patch<8, 8><<<patch_blocks<8, 8>(), PATCH_NT, 0, s>>>(sc.probs, sc.tbase, o);  // no pairs: fan search
     SDF_LAUNCHED(1);
     SDF_TRY(cudaGetLastError());
     if (sc.fprobs)
