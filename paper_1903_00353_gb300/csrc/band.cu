@@ -200,6 +200,53 @@ __device__ __forceinline__ float cone_reach(float ca, float cth, float sth) {
     return fmaxf(0.f, ca * cth + sa * sth);  // cos(angle(e, axis) - theta), or the apex
 }
 
+// Whether a thin region may hold a grid point: on a smooth, finely tessellated mesh the wedge of an
+// edge and the cone of a vertex are needles along the surface normal that mostly pass between the
+// grid points, and setting them up in the tile kernel costs as much as a region with points.
+// The region lies within s T + r n + e of the point `fa`, 0 <= s <= 1, with n its axis and e, in a layer
+// of the grid across n's largest component, at most `tol` per axis (all in cells).  Per layer of the
+// region's integer box that leaves a small parallelogram, whose grid points are tested.  `tol` covers
+// the inclusion tolerance, the rounding of the row spans and their slack, so a region without a point
+// here is one whose row spans are all empty; the others keep their box, since its sides choose the
+// scan axis and so the rounding of the spans.  On the 2.1 M-triangle knot at 512^3 this drops 9 of 10
+// edge and nearly all vertex regions (9.6 to 6.2 M (tile, region) pairs, 43.9 to 29.4 M rows, the tile
+// kernel 896 to 689 us, against 40 us more in the count pass of the binning).  Regions of more than THIN_TOL cells' width or THIN_LEN cells' length hold points anyway and are not tested.
+constexpr float THIN_LEN = 4.f, THIN_TOL = 0.5f, THIN_REACH = 16.f;  // cells
+constexpr int THIN_GRID = 4096;  // longest grid axis: the index rounding stays below 1/1024 cell
+__device__ __forceinline__ bool thin_holds_point(float3 fa, float3 n, float3 T, float tol, int i0, int i1, int j0,
+                                                 int j1, int k0, int k1) {
+    const float ax = fabsf(n.x), ay = fabsf(n.y), az = fabsf(n.z);
+    const int la = (ax >= ay && ax >= az) ? 0 : (ay >= az ? 1 : 2);  // layers across this axis, (b, c) in a layer
+    const float inv = 1.f / (la == 0 ? n.x : (la == 1 ? n.y : n.z));
+    const float fa_a = la == 0 ? fa.x : (la == 1 ? fa.y : fa.z), Ta = la == 0 ? T.x : (la == 1 ? T.y : T.z);
+    const float fb = la == 0 ? fa.y : fa.x, fc = la == 2 ? fa.y : fa.z;
+    const float sb = (la == 0 ? n.y : n.x) * inv, sc = (la == 2 ? n.y : n.z) * inv;
+    const float Tb = (la == 0 ? T.y : T.x) - Ta * sb, Tc = (la == 2 ? T.y : T.z) - Ta * sc;
+    const int a0 = la == 0 ? i0 : (la == 1 ? j0 : k0), a1 = la == 0 ? i1 : (la == 1 ? j1 : k1);
+    const int b0 = la == 0 ? j0 : i0, b1 = la == 0 ? j1 : i1, c0 = la == 2 ? j0 : k0, c1 = la == 2 ? j1 : k1;
+    const float blo = fminf(Tb, 0.f) - tol, bhi = fmaxf(Tb, 0.f) + tol, clo = fminf(Tc, 0.f) - tol,
+                chi = fmaxf(Tc, 0.f) + tol, strip = (fabsf(Tb) + fabsf(Tc)) * tol;
+    for (int a = a0; a <= a1; a++) {
+        const float rel = (float)a - fa_a, pb = fmaf(rel, sb, fb), pc = fmaf(rel, sc, fc);
+        const int p0 = max((int)ceilf(pb + blo), b0), p1 = min((int)floorf(pb + bhi), b1);
+        const int q0 = max((int)ceilf(pc + clo), c0), q1 = min((int)floorf(pc + chi), c1);
+        for (int p = p0; p <= p1; p++)
+            for (int q = q0; q <= q1; q++)
+                if (fabsf(Tc * ((float)p - pb) - Tb * ((float)q - pc)) <= strip) return true;
+    }
+    return false;
+}
+__device__ __forceinline__ bool thin_grid(const GridP &g) {
+    return max(max(g.nx, g.ny), g.kofs + g.nz) <= THIN_GRID && (g.W + g.eps) * g.inv_h <= THIN_REACH;
+}
+// what a row span may add to a region, in world units: the inclusion tolerance, the rounding of the
+// span's bounds and of the region's planes (delta each), and the slack of 1/4096 cell
+__device__ __forceinline__ float span_tol(const GridP &g) { return g.eps + 2.f * g.derr + g.h * (1.f / 2048.f); }
+__device__ __forceinline__ float3 to_index(const GridP &g, float4 p) {
+    return make_float3((p.x - g.ox) * g.inv_h - 0.5f, (p.y - g.oy) * g.inv_h - 0.5f,
+                       (p.z - g.oz) * g.inv_h - 0.5f - (float)g.kofs);
+}
+
 // integer box of the clipped region of feature `id` of type TYPE; false if the feature has none.
 //   face  : triangle box grown by W |n| per axis (the prism is the triangle swept along +-W n);
 //   edge  : segment box plus the box of the sector of radius W between the two face normals
@@ -235,24 +282,53 @@ __device__ __forceinline__ bool feature_box(const Feat &F, const GridP &g, int i
             shi = make_float3(1.f, 1.f, 1.f);
         }
         const float bx = fmaf(a.w, t.x, a.x), by = fmaf(a.w, t.y, a.y), bz = fmaf(a.w, t.z, a.z);
-        return to_index_box(fminf(a.x, bx) + R * slo.x - slack, fminf(a.y, by) + R * slo.y - slack,
-                            fminf(a.z, bz) + R * slo.z - slack, fmaxf(a.x, bx) + R * shi.x + slack,
-                            fmaxf(a.y, by) + R * shi.y + slack, fmaxf(a.z, bz) + R * shi.z + slack, g, i0, i1, j0,
-                            j1, k0, k1);
+        if (!to_index_box(fminf(a.x, bx) + R * slo.x - slack, fminf(a.y, by) + R * slo.y - slack,
+                          fminf(a.z, bz) + R * slo.z - slack, fmaxf(a.x, bx) + R * shi.x + slack,
+                          fmaxf(a.y, by) + R * shi.y + slack, fmaxf(a.z, bz) + R * shi.z + slack, g, i0, i1, j0, j1,
+                          k0, k1))
+            return false;
+        // the wedge is a + s t + r n + q (t x n) with n the unit mean normal, 0 <= r <= R and
+        // |q| <= r tan(theta / 2); a point of a layer moves by at most sqrt(2) |q| per axis with q, and
+        // by sqrt(2) times the tolerance along t
+        if (!thin_grid(g) || lm <= 1.f || a.w * g.inv_h > THIN_LEN) return true;
+        const float c2 = 0.25f * lm * lm;  // cos^2(theta / 2); 1 - c2 errs by a few u
+        const float tol = 1.5f * (R * sqrtf(fmaxf(1.f - c2, 0.f) + 1e-6f) / sqrtf(c2) + 2.f * span_tol(g)) * g.inv_h +
+                          1.f / 1024.f;
+        if (tol > THIN_TOL) return true;
+        const float len = a.w * g.inv_h;
+        return thin_holds_point(to_index(g, a), (1.f / lm) * ms, len * tt, tol, i0, i1, j0, j1, k0, k1);
     } else {
         const int8_t c = F.vert_class[id];
         if (c == CLS_FLAT || (F.skip_saddle && c == CLS_SADDLE)) return false;
-        const float4 v = __ldg(F.vert_rec + 3 * id), cone = __ldg(F.vert_rec + 3 * id + 2);
+        // (axis sign, needle slope, 1 / needle width bound, cos or -(2 + 1 / mu)); see k_vertex_records
+        const float4 v = __ldg(F.vert_rec + 3 * id), nv = __ldg(F.vert_rec + 3 * id + 1),
+                     cn = __ldg(F.vert_rec + 3 * id + 2);
         float3 lo = make_float3(-1.f, -1.f, -1.f), hi = make_float3(1.f, 1.f, 1.f);
-        if (cone.w > -1.f) {
-            const float cth = fminf(cone.w, 1.f), sth = sqrtf(fmaxf(0.f, 1.f - cth * cth));
+        if (cn.w > -1.f) {
+            const float3 cone = cn.x * f3(nv);
+            const float cth = fminf(cn.w, 1.f), sth = sqrtf(fmaxf(0.f, 1.f - cth * cth));
             hi = make_float3(cone_reach(cone.x, cth, sth), cone_reach(cone.y, cth, sth), cone_reach(cone.z, cth, sth));
             lo = make_float3(-cone_reach(-cone.x, cth, sth), -cone_reach(-cone.y, cth, sth),
                              -cone_reach(-cone.z, cth, sth));
         }
-        return to_index_box(v.x + R * lo.x - slack, v.y + R * lo.y - slack, v.z + R * lo.z - slack,
-                            v.x + R * hi.x + slack, v.y + R * hi.y + slack, v.z + R * hi.z + slack, g, i0, i1, j0,
-                            j1, k0, k1);
+        if (!to_index_box(v.x + R * lo.x - slack, v.y + R * lo.y - slack, v.z + R * lo.z - slack,
+                          v.x + R * hi.x + slack, v.y + R * hi.y + slack, v.z + R * hi.z + slack, g, i0, i1, j0, j1,
+                          k0, k1))
+            return false;
+        if (cn.w < -2.f) {
+            // no direction leads away from every neighbour: the region is the vertex alone, and with the
+            // half-spaces moved out by a tolerance it stays within tolerance / mu of it
+            const float Rv = 1.01f * span_tol(g) * (-2.f - cn.w) + 1e-3f * g.h;
+            int a0, a1, b0, b1, c0, c1;
+            if (!to_index_box(v.x - Rv, v.y - Rv, v.z - Rv, v.x + Rv, v.y + Rv, v.z + Rv, g, a0, a1, b0, b1, c0, c1))
+                return false;
+        }
+        if (!thin_grid(g) || !(cn.z > 0.f)) return true;
+        // the needle: at distance r along N_alpha, points within r slope (+ tolerance / width bound) of the axis
+        const float na = fmaxf(fmaxf(fabsf(nv.x), fabsf(nv.y)), fabsf(nv.z));
+        const float tol = (R * cn.y + span_tol(g) * cn.z) * g.inv_h / na * 1.01f + 1.f / 1024.f;
+        if (tol > THIN_TOL) return true;
+        return thin_holds_point(to_index(g, v), f3(nv), make_float3(0.f, 0.f, 0.f), tol, i0, i1, j0, j1, k0, k1);
     }
 }
 
@@ -290,17 +366,29 @@ __device__ __forceinline__ int warp_owner(int incl, int r) {
     return lo;
 }
 
+// ----------------------------------------------------------------------------- type dispatch
+__device__ __forceinline__ int feat_type(const Feat &F, int fid) { return fid < F.T ? FACE : (fid < F.T + F.E ? EDGE : VERT); }
+__device__ __forceinline__ int feat_local(const Feat &F, int fid, int type) {
+    return type == FACE ? fid : (type == EDGE ? fid - F.T : fid - F.T - F.E);
+}
+
 // Binning of the regions into tiles, one thread per feature, its (feature, tile) pairs flattened
 // over the warp: in each round every lane takes one pair, lanes whose pairs fall in the same bin
 // (neighbouring features share tiles: faces, edges and vertices are numbered in spatial order)
 // are grouped by __match_any_sync, and one atomic per group takes their slots.  The count pass
-// (FILL false) and the fill pass walk the same pairs; the fill pass takes each bin's slots by
+// (BIN_COUNT) and the fill pass walk the same pairs; the fill pass takes each bin's slots by
 // counting its count back down to 0 (so the counts need no clearing in between, and end cleared).
-template <bool FILL, int TY, int TZ>
+// The count pass leaves the features' boxes in `boxes` (12 bytes a feature), where the fill pass reads
+// them instead of the records (48 to 96 bytes) and the arithmetic; without the array (a grid of more
+// than 65536 points along an axis, the allocation-free entry point) BIN_FILL_AGAIN works them out again.
+enum { BIN_COUNT = 0, BIN_FILL = 1, BIN_FILL_AGAIN = 2 };
+template <int MODE, int TY, int TZ>
 __global__ void k_bin(const Prob *P, const long long *feat_base, const long long *tile_base, int n, long long f_tot,
-                      uint32_t *cnt, const uint32_t *start, int2 *pairs, int64_t pair_cap, DevCounters *ctr) {
+                      uint32_t *cnt, const uint32_t *start, int2 *pairs, int64_t pair_cap, DevCounters *ctr,
+                      uint32_t *boxes) {
     dep_wait();
     dep_next();
+    constexpr bool FILL = MODE != BIN_COUNT;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     int p = 0, type = 0, fid = 0, ntile = 0;
@@ -311,11 +399,25 @@ __global__ void k_bin(const Prob *P, const long long *feat_base, const long long
         const GridP &g = P[p].g;
         const int64_t lid = gid - feat_base[p];
         bool ok;
-        int id;
-        if (lid < F.T) { type = FACE; id = (int)lid; ok = feature_box<FACE>(F, g, id, i0, i1, j0, j1, k0, k1); }
-        else if (lid < (int64_t)F.T + F.E) { type = EDGE; id = (int)(lid - F.T); ok = feature_box<EDGE>(F, g, id, i0, i1, j0, j1, k0, k1); }
-        else { type = VERT; id = (int)(lid - F.T - F.E); ok = feature_box<VERT>(F, g, id, i0, i1, j0, j1, k0, k1); }
+        type = lid < F.T ? FACE : (lid < (int64_t)F.T + F.E ? EDGE : VERT);
+        if (MODE == BIN_FILL) {
+            const uint32_t bi = boxes[gid], bj = boxes[f_tot + gid], bk = boxes[2 * f_tot + gid];
+            i0 = (int)(bi & 0xffffu); i1 = (int)(bi >> 16);
+            j0 = (int)(bj & 0xffffu); j1 = (int)(bj >> 16);
+            k0 = (int)(bk & 0xffffu); k1 = (int)(bk >> 16);
+            ok = i0 <= i1;
+        } else {
+            const int id = feat_local(F, (int)lid, type);
+            if (type == FACE) ok = feature_box<FACE>(F, g, id, i0, i1, j0, j1, k0, k1);
+            else if (type == EDGE) ok = feature_box<EDGE>(F, g, id, i0, i1, j0, j1, k0, k1);
+            else ok = feature_box<VERT>(F, g, id, i0, i1, j0, j1, k0, k1);
+        }
         fid = (int)lid;  // face f -> f, edge e -> T + e, vertex v -> T + E + v (within its problem)
+        if (MODE == BIN_COUNT && boxes) {
+            boxes[gid] = ok ? (uint32_t)i0 | (uint32_t)i1 << 16 : 1u;  // (1, 0): no box
+            boxes[f_tot + gid] = (uint32_t)j0 | (uint32_t)j1 << 16;
+            boxes[2 * f_tot + gid] = (uint32_t)k0 | (uint32_t)k1 << 16;
+        }
         if (ok)
             ntile = (i1 / TILE_X - i0 / TILE_X + 1) * (j1 / TY - j0 / TY + 1) * (k1 / TZ - k0 / TZ + 1);
     }
@@ -415,11 +517,6 @@ __device__ __forceinline__ float eval_point(const Feat &F, const GridP &g, int i
     }
 }
 
-// ----------------------------------------------------------------------------- type dispatch
-__device__ __forceinline__ int feat_type(const Feat &F, int fid) { return fid < F.T ? FACE : (fid < F.T + F.E ? EDGE : VERT); }
-__device__ __forceinline__ int feat_local(const Feat &F, int fid, int type) {
-    return type == FACE ? fid : (type == EDGE ? fid - F.T : fid - F.T - F.E);
-}
 __device__ __forceinline__ float eval_any(const Feat &F, const GridP &g, int type, int id, int i, int j, int k,
                                           bool &neg, bool &unc) {
     if (type == FACE) return eval_point<FACE>(F, g, id, i, j, k, neg, unc);
@@ -2096,10 +2193,11 @@ struct Plan {
     int vmode = VM_EXACT;
     std::vector<long long> pbase;
     long long p_tot = 0;
-    DevBuf tables, bins, pairs, patch, scan_tmp, lists, rowsign, keys, split;
+    DevBuf tables, bins, pairs, patch, scan_tmp, lists, rowsign, keys, split, boxes;
     DevCounters *ctr = nullptr;
     bool own_ctr = false;
     int64_t pair_cap = 0, patch_cap = 0;
+    bool small_dims = true;  // no grid axis has more than 65536 points: boxes fit 16-bit indices
     int64_t pair_est = 0;  // expected (tile, region) pairs of the described problems (pair_estimate)
     double tuned_ms = 0.0;
     sdf_features_s *events = nullptr;  // handle whose events time the stages (SDF_FLAG_TIMING)
@@ -2151,6 +2249,7 @@ void plan_free(Plan *pl, cudaStream_t s) {
     pl->tables.release(s);
     pl->bins.release(s);
     pl->pairs.release(s);
+    pl->boxes.release(s);
     pl->patch.release(s);
     pl->split.release(s);
     pl->scan_tmp.release(s);
@@ -2236,6 +2335,7 @@ static int plan_describe(Plan &pl, const sdf_features *feats, const sdf_grid *gr
     pl.ybase.assign(n + 1, 0);
     pl.pbase.assign(n + 1, 0);
     pl.pair_est = 0;
+    pl.small_dims = true;
     for (int p = 0; p < n; p++) {
         // the dense field may be left out only by a sparse forward (a list with its distances)
         const bool sparse = lists && lists[p].list && lists[p].dist;
@@ -2243,6 +2343,7 @@ static int plan_describe(Plan &pl, const sdf_features *feats, const sdf_grid *gr
         Prob &pr = pl.probs[p];
         int st = make_grid(grids[p], band_w[p], shape, pr.g);
         if (st) return st;
+        pl.small_dims = pl.small_dims && std::max(grids[p].nx, std::max(grids[p].ny, grids[p].nz)) <= 65536;
         pr.F = make_feat(feats[p]);
         pr.F.vmode = pl.vmode;
         pl.pair_est += pair_estimate(feats[p], pr.g, shape);
@@ -2299,6 +2400,7 @@ static int plan_reserve(Plan &pl, cudaStream_t s) {
     const size_t tb = sizeof(Prob) * pl.n + 2 * sizeof(long long) * (pl.n + 1) + sizeof(FillProb) * pl.n +
                       4 * sizeof(long long) * (pl.n + 1) + 256;
     SDF_TRY(pl.tables.reserve(tb, s));
+    if (!pl.cell_loop && pl.small_dims) SDF_TRY(pl.boxes.reserve(3 * sizeof(uint32_t) * (size_t)pl.f_tot, s));
     if (pl.fill) SDF_TRY(pl.rowsign.reserve((size_t)pl.r_tot + 64, s));
     if (pl.cell_loop) SDF_TRY(pl.keys.reserve(sizeof(unsigned long long) * (size_t)pl.p_tot, s));
     SDF_TRY(pl.bins.reserve(sizeof(uint32_t) * (size_t)(2 * n_bins + 64), s));
@@ -2382,6 +2484,7 @@ struct Scratch {  // device pointers used by one launch of the pipeline
     int32_t *band_list, *empty_list;
     int2 *pairs;
     int64_t pair_cap;
+    uint32_t *boxes = nullptr;  // the features' integer boxes (nullable, see k_bin)
     PatchEntry *patch;
     int64_t patch_cap;
     DevCounters *ctr;
@@ -2436,6 +2539,7 @@ static Scratch plan_scratch(const Plan &pl) {
     sc.empty_list = sc.band_list + pl.n_tiles + 32;
     sc.pairs = pl.pairs.as<int2>();
     sc.pair_cap = pl.pair_cap;
+    sc.boxes = pl.small_dims ? pl.boxes.as<uint32_t>() : nullptr;
     sc.patch = pl.patch.as<PatchEntry>();
     sc.patch_cap = pl.patch_cap;
     sc.ctr = pl.ctr;
@@ -2459,11 +2563,11 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
         SDF_TRY(launch_dep(k_front, dim3(blocks), dim3(256), 0, s, const_cast<Prob *>(sc.probs), n, sc.cnt, n_bins,
                            sc.ctr, sc.ticket, sc.split_items ? 3 : 2));
     }
-    SDF_TRY(launch_dep(k_bin<false, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
-                       f_tot, sc.cnt, (const uint32_t *)nullptr, (int2 *)nullptr, (int64_t)0, sc.ctr));
+    SDF_TRY(launch_dep(k_bin<BIN_COUNT, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
+                       f_tot, sc.cnt, (const uint32_t *)nullptr, (int2 *)nullptr, (int64_t)0, sc.ctr, sc.boxes));
     SDF_TRY(scan_exclusive_u32(sc.cnt, sc.start, n_bins, true, sc.scan_tmp, s, &sc.ctr->nb_status));
-    SDF_TRY(launch_dep(k_bin<true, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
-                       f_tot, sc.cnt, (const uint32_t *)sc.start, sc.pairs, sc.pair_cap, sc.ctr));
+    SDF_TRY(launch_dep(sc.boxes ? k_bin<BIN_FILL, TY, TZ> : k_bin<BIN_FILL_AGAIN, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
+                       f_tot, sc.cnt, (const uint32_t *)sc.start, sc.pairs, sc.pair_cap, sc.ctr, sc.boxes));
     // band / empty tile lists for the persistent tile kernel (one scan of the band flags)
     uint32_t *flags = sc.cnt;  // the fill cursors are no longer needed
     const int lpt = n > 1;  // largest-first order of the band tiles for batches

@@ -521,6 +521,7 @@ __device__ __forceinline__ float corner_angle(float3 e1, float3 e2) {
 
 constexpr int VL = 8;      // lanes per vertex in k_vertex_records
 constexpr int VMAXS = 24;  // corners of a fan staged in shared memory (and cone-searched)
+constexpr int NARROW_VP = 6;  // planes of a vertex region that the narrow band tests (MAXVP in band.cu)
 
 __device__ __forceinline__ float gsum8(float v) {
     v += __shfl_xor_sync(0xffffffffu, v, 4, VL);
@@ -628,7 +629,7 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         const float3 p = valid ? load_vpos(vpos, (int)v) : make_float3(0.f, 0.f, 0.f);
         // pass 1: pseudonormal and region planes
         float3 N = make_float3(0.f, 0.f, 0.f);
-        float asum = 0.f;
+        float asum = 0.f, amax = 0.f, zmax = 0.f;
         const bool staged = s1 - s0 <= VMAXS;  // the fan's planes and normals fit the group's slots
         for (int i = s0 + sub; i < s1; i += VL) {
             const int c = vert_corner[i];
@@ -638,6 +639,7 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
             const float3 e1 = xn - p, e2 = xp - p;
             const float alpha = corner_angle(e1, e2);
             asum += alpha;
+            amax = fmaxf(amax, alpha);
             const float3 nf = f3(face_rec[4 * f]);
             N = N + alpha * nf;
             const float3 ej = normalized(e1);
@@ -650,6 +652,7 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         }
         N = make_float3(gsum8(N.x), gsum8(N.y), gsum8(N.z));
         asum = gsum8(asum);
+        amax = -gmin8(-amax);
         const float Nlen = sqrtf(dot3(N, N));
         const float3 Nu = (Nlen > 0.f ? 1.f / Nlen : 0.f) * N;
         // Direction error of the unit pseudonormal: each term alpha_i n_i errs by at most
@@ -665,13 +668,14 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         }
         __syncwarp();  // the group's planes are written before they are read back
         // pass 2: classification (FP32 with an error margin), convexity and the normal spread
-        bool below = false, above = false, unsure = false, cvx = true, ccv = true;
-        float cmin = 1.f;
+        bool below = false, above = false, unsure = false;
+        float cmin = 1.f, ddlo = 0.f, ddhi = 0.f;
         for (int i = s0 + sub; i < s1; i += VL) {
             // unit direction e_j to the next neighbour (the plane holds -e_j): the sign of
             // (v_n - v).N_alpha is that of e_j.N_alpha, tested against 2e-6 |N_alpha|
             const float3 ej = -1.f * (staged ? f3(s_plane[grp][i - s0]) : f3(vert_plane[i]));
             const float d = dot3(ej, N);
+            zmax = fmaxf(zmax, fabsf(d));
             const float bound = 2e-6f * Nlen;
             if (d < -bound) below = true;
             else if (d > bound) above = true;
@@ -680,16 +684,16 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
             cmin = fminf(cmin, dot3(nf, Nu));
             for (int b = 0; b < s1 - s0; b++) {  // every incident edge against this face's plane
                 const float dd = -dot3(nf, staged ? f3(s_plane[grp][b]) : f3(vert_plane[s0 + b]));
-                cvx = cvx && dd <= 1e-4f;
-                ccv = ccv && dd >= -1e-4f;
+                ddlo = fminf(ddlo, dd);
+                ddhi = fmaxf(ddhi, dd);
             }
         }
         below = gor8(below);
         above = gor8(above);
         unsure = gor8(unsure);
-        cvx = !gor8(!cvx);
-        ccv = !gor8(!ccv);
+        const bool cvx = !gor8(ddhi > 1e-4f), ccv = !gor8(ddlo < -1e-4f);
         cmin = gmin8(cmin);
+        zmax = -gmin8(-zmax);
         // Bound of the vertex region {y : y.e_j <= 0}.  Locally convex (every incident edge below every
         // incident face plane): the cone spanned by the face normals; locally concave: by their
         // negatives; otherwise the extreme rays are searched among +-(e_j x e_l): the deg (deg - 1) / 2
@@ -697,30 +701,43 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         // every plane without early exit, so the lanes of a group stay converged.  A cone is kept only
         // if all its rays lie within 89 degrees of +N_alpha (or of -N_alpha).  The flags and bounds
         // below are uniform over the 8 lanes of a vertex after the group reductions.
+        // Two more bounds tell the narrow band which regions hold no grid point (feature_box); the tile
+        // kernel tests a vertex's first NARROW_VP planes, so both are left out for larger fans.
+        //  - No feasible ray: the region is v alone, and {y : y.e_j <= t} lies within t / mu of it, mu the
+        //    distance of the hull of the e_j from the origin inside it.  At the nearest facet (a, b, c),
+        //    u.e_a = u.e_b = u.e_c = mu with u its normal; some two of them, a and b, are at most 120 degrees
+        //    apart, u = cos(f) y + sin(f) w with y = +-(e_a x e_b) / |..| and w their bisector, w.e_a = k >= 1/2,
+        //    sin(f) = mu / k.  For the e_m that ray y violates most, by v, cos(f) v <= u.e_m - sin(f) w.e_m
+        //    <= mu (1 + 1 / k), so mu >= cos(f) v / 3 > v / 4.  viol is the smallest v over the pairs of at
+        //    most 127 degrees (0 where a pair is too close to parallel to give y).
+        //  - The region is a needle along N_alpha where the fan is nearly flat: with the neighbours' heights
+        //    |e_j.N^| <= z and the gaps between consecutive tangential directions at most g (the fan's
+        //    corners, all facing N_alpha and turning once: cmin > 0.9, sum of angles < 3 pi), every
+        //    tangential direction has an e_j at most g / 2 away, so y with y.e_j <= t has a tangential part
+        //    of at most (t + z |y.N^|) / width, width = cos(g / 2) sqrt(1 - z^2).
         const int deg = s1 - s0;
         const bool conv_cone = cvx && !ccv && cmin > 0.02f, conc_cone = ccv && !cvx && cmin > 0.02f;
         const bool search = valid && Nlen > 0.f && !conv_cone && !conc_cone && staged;
         bool any = false, all_pos = true, all_neg = true;
-        float cpos = 1.f, cng = 1.f;
+        float cpos = 1.f, cng = 1.f, viol = 1.f;
         if (search) {
             const int npairs = deg * (deg - 1) / 2;
             for (int pidx = sub; pidx < npairs; pidx += VL) {
-                int a = 0, rem = pidx;  // pair pidx = (a, b), a < b, in row-major order
-                while (rem >= deg - 1 - a) {
-                    rem -= deg - 1 - a;
-                    a++;
-                }
-                const int b = a + 1 + rem;
+                const int b = (int)(0.5f * (1.f + sqrtf((float)(8 * pidx + 1))));  // pidx = b (b - 1) / 2 + a, a < b
+                const int a = pidx - b * (b - 1) / 2;
                 float3 y = cross3(f3(s_plane[grp][a]), f3(s_plane[grp][b]));  // planes hold -e
                 const float ly = sqrtf(dot3(y, y));
                 const bool ok = ly > 1e-6f;
                 y = (ok ? 1.f / ly : 0.f) * y;
-                bool fp = ok, fn = ok;  // +y and -y feasible
+                float dlo = 0.f, dhi = 0.f;  // smallest and largest value of -e.y over the planes (0 at a and b)
                 for (int m = 0; m < deg; m++) {
                     const float dm = dot3(y, f3(s_plane[grp][m]));
-                    fp = fp && dm >= -1e-4f;
-                    fn = fn && -dm >= -1e-4f;
+                    dlo = fminf(dlo, dm);
+                    dhi = fmaxf(dhi, dm);
                 }
+                const bool fp = ok && dlo >= -1e-4f, fn = ok && dhi <= 1e-4f;  // +y and -y feasible
+                const float eab = dot3(f3(s_plane[grp][a]), f3(s_plane[grp][b]));
+                if (eab > -0.6f) viol = fminf(viol, ly > 0.05f ? fminf(-dlo, dhi) : 0.f);
                 const float cc = dot3(y, Nu);
                 if (fp) {
                     any = true;
@@ -739,6 +756,7 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         all_neg = !gor8(!all_neg);
         cpos = gmin8(cpos);
         cng = gmin8(cng);
+        viol = gmin8(viol);
         if (__any_sync(0xffffffffu, unsure))  // FP64 filtered predicate
             classify64(unsure, vert_corner, face_vid, vpos, s0, s1, p, below, above);
         int8_t my_cls = 99;  // class of the vertex held by lane sub == 0
@@ -747,10 +765,20 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
             vert_class[v] = cls;
             float4 cone = make_float4(0.f, 0.f, 0.f, -2.f);
             if (Nlen > 0.f) {
-                if (conv_cone) cone = make_float4(Nu.x, Nu.y, Nu.z, cmin - 2e-3f);
-                else if (conc_cone) cone = make_float4(-Nu.x, -Nu.y, -Nu.z, cmin - 2e-3f);
-                else if (search && any && all_pos) cone = make_float4(Nu.x, Nu.y, Nu.z, cpos - 2e-3f);
-                else if (search && any && all_neg) cone = make_float4(-Nu.x, -Nu.y, -Nu.z, cng - 2e-3f);
+                if (conv_cone) cone = make_float4(1.f, 0.f, 0.f, cmin - 2e-3f);
+                else if (conc_cone) cone = make_float4(-1.f, 0.f, 0.f, cmin - 2e-3f);
+                else if (search && any && all_pos) cone = make_float4(1.f, 0.f, 0.f, cpos - 2e-3f);
+                else if (search && any && all_neg) cone = make_float4(-1.f, 0.f, 0.f, cng - 2e-3f);
+                else if (search && !any && deg <= NARROW_VP && viol > 1e-3f) cone.w = -2.f - 4.f / viol;
+                if (deg <= NARROW_VP && cmin > 0.9f && asum < 9.42f) {
+                    const float z = zmax / Nlen * 1.001f + 1e-5f, z2 = fminf(z * z, 0.5f);
+                    const float ca = cospif(0.318309886f * amax) - 1e-5f - z2, cg = fmaxf(ca < 0.f ? ca / (1.f - z2) : ca, -1.f);
+                    const float width = 0.999f * sqrtf(0.5f * (1.f + cg) * (1.f - z2));
+                    if (width > 0.2f) {
+                        cone.y = z / width;
+                        cone.z = 1.f / width;
+                    }
+                }
             }
             vert_rec[3 * v + 0] = make_float4(p.x, p.y, p.z, __int_as_float(s0));
             vert_rec[3 * v + 1] = make_float4(Nu.x, Nu.y, Nu.z, __int_as_float(s1 - s0));
