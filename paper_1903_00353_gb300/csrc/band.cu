@@ -20,11 +20,10 @@
 //      default; 4x4 and 16x8 for the autotuner) and the (tile, region) pairs, each with the
 //      region's box clipped to the tile, are bucketed per tile and type (count, scan, fill;
 //      a warp's pairs share one atomic per bin); tiles of all problems share one numbering;
-//   2. tile kernel: a persistent grid (4 CTAs of 256 threads per SM) takes work items from one
-//      atomic ticket: a band tile plus its share of the empty tiles (band tiles largest first
-//      for batches).  A band tile keeps the packed keys (|d| bits << 32 | id << 1 | sign) of
-//      its points in shared memory.  Warps take chunks of at most 32 of the tile's regions
-//      without block barriers: one lane per region computes its scan axis and per-plane span
+//   2. tile kernel: a persistent grid (6 CTAs of 128 threads per SM, or 4 of 256 on small grids)
+//      takes work items from two atomic tickets, the band tiles (largest first for batches) and
+//      chunks of the empty tiles.  A band tile keeps the packed keys (|d| bits << 32 | id << 1 | sign) of
+//      its points in shared memory.  One lane per region computes its scan axis and per-plane span
 //      coefficients (Algorithm 2 restricted to grid lines, with the inclusion tolerance of
 //      Section 10), a warp scan numbers the rows, each lane evaluates one row's span, and the
 //      span points are flattened across lanes, evaluated against the feature and merged with a
@@ -52,7 +51,6 @@ namespace sdf {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int NT = 256;  // threads per tile CTA (and regions per pass)
 enum { FACE = 0, EDGE = 1, VERT = 2 };
 
 struct GridP {
@@ -461,7 +459,6 @@ __global__ void k_bin(const Prob *P, const long long *feat_base, const long long
     }
 }
 
-__device__ __forceinline__ float comp(float4 P, int ax) { return ax == 0 ? P.x : (ax == 1 ? P.y : P.z); }
 __device__ __forceinline__ float comp3(float3 P, int ax) { return ax == 0 ? P.x : (ax == 1 ? P.y : P.z); }
 
 // FP32 distance to the triangle boundary (three clamped segments); used for points of the face
@@ -541,173 +538,217 @@ __device__ __forceinline__ float eval_any(const Feat &F, const GridP &g, int typ
 // region, and a point outside the exact vertex region has a strictly closer point on an incident
 // edge.  Faces have 5 planes, edges 4.
 constexpr int KMAX = 6, MAXVP = 6;
-constexpr float Q_NONE = 0.f, Q_EDGE = 1.f, Q_VERT = 2.f;  // kinds of quadratic row bound
+enum { Q_NONE = 0, Q_EDGE = 1, Q_VERT = 2 };  // kinds of quadratic row bound
 
-template <int TY, int TZ>
+template <int TY, int TZ, int NT>
 struct TileSmem {
     unsigned long long key[TILE_X * TY * TZ];  // packed (|d| bits << 32 | id << 2 | unc << 1 | neg) per point
     float4 coef[NT][KMAX];             // span coefficients (A, B, C, -): nl lower bounds, then upper bounds
     float4 quad[NT][2];                // quadratic bound of a region's rows: vertex ball, edge cylinder
     uint2 rinfo[NT];                   // row set-up of each region, packed (see setup_region)
     int fid[NT];                       // regions of the current pass (global feature ids)
-    unsigned char ax[NT];              // scan axis
-    unsigned char qkind[NT];           // kind of quadratic row bound: Q_NONE, Q_EDGE or Q_VERT
-    unsigned rowq[NT / 32][64];        // per-warp ring of non-empty rows waiting for point evaluation
+    unsigned char axq[NT];             // scan axis | kind of quadratic row bound (Q_NONE, Q_EDGE or Q_VERT) << 2
+    unsigned short pre[NT + NT / 32]; // first row of each region, per pass or per warp (see process_band_tile)
+    int wsum[NT / 32];                 // rows of each warp's regions
+    uint2 rowq[NT / 32][64];           // per-warp ring of non-empty rows waiting for point evaluation
     int next;                          // next chunk of the tile's regions to hand to a warp
     long long work;
 };
 
 
 
-__device__ __forceinline__ void add_coef(float4 *E, int &nl, int &nu, float4 P, int ax, int bx, int cx, float pb0,
-                                         float pc0, float K, const GridP &g) {
-    const float ma = comp(P, ax), mb = comp(P, bx), mc = comp(P, cx);
-    const float r0 = fmaf(mb, pb0, fmaf(mc, pc0, P.w)) + g.eps;
-    if (ma > 0.f) {
-        const float inv = 1.f / ma;
-        E[nl++] = make_float4(fmaf(-r0 * inv, g.inv_h, -K), -mb * inv, -mc * inv, 0.f);
-    } else if (ma < 0.f) {
-        const float inv = 1.f / ma;
-        E[KMAX - 1 - nu++] = make_float4(fmaf(-r0 * inv, g.inv_h, -K), -mb * inv, -mc * inv, 0.f);
-    } else {
-        const float s = -0x1p100f;
-        E[nl++] = make_float4(s * r0, s * (mb * g.h), s * (mc * g.h), 0.f);
-    }
+// The components of a plane along a region's scan axis and its two other axes (in order).
+__device__ __forceinline__ float3 along(float4 P, int ax) {
+    return make_float3(ax == 0 ? P.x : (ax == 1 ? P.y : P.z), ax == 0 ? P.y : P.x, ax == 2 ? P.y : P.z);
 }
 
-// Points of n (<= 32) queued rows, starting at ring slot q0, flattened over the lanes of the warp:
-// distance to the row's feature, and the merge into the tile's keys (Algorithm 1).
-template <int TY, int TZ>
-__device__ __forceinline__ void eval_rows(const Feat &F, const GridP &g, TileSmem<TY, TZ> &S, const unsigned *Q,
-                                          int q0, int n, int x0, int y0, int z0, unsigned &cand) {
-    const int lane = threadIdx.x & 31;
-    const unsigned e = lane < n ? Q[(q0 + lane) & 63] : 0u;
-    const int len = (int)((e >> 13) & 63u);
-    const int pincl = warp_incl_scan(len);
-    const int ptotal = __shfl_sync(FULL, pincl, 31);
-    for (int p0 = 0; p0 < ptotal; p0 += 32) {
-        const int pp = p0 + lane;
-        const int ro = min(warp_owner(pincl, pp), 31);
-        const unsigned re = __shfl_sync(FULL, e, ro);
-        const int rfirst = __shfl_sync(FULL, pincl - len, ro);  // points before this row
-        if (pp < ptotal) {
-            const int slot = (int)(re & 255u);
-            const int la = (int)((re >> 8) & 31u) + (pp - rfirst), lb = (int)((re >> 19) & 31u), lc = (int)((re >> 24) & 31u);
-            const int ax = S.ax[slot];
-            const int lx = ax == 0 ? la : lb;
-            const int ly = ax == 1 ? la : (ax == 0 ? lb : lc);
-            const int lz = ax == 2 ? la : lc;
-            const int fid = S.fid[slot];
-            const int type = feat_type(F, fid), id = feat_local(F, fid, type);
-            bool neg, unc;
-            const float d = eval_any(F, g, type, id, x0 + lx, y0 + ly, z0 + lz, neg, unc);
-            if (d < g.W) {
-                atomicMin(S.key + (lz * TY + ly) * TILE_X + lx, make_key(d, fid, unc, neg));
-                cand++;
-            }
+// What the row coefficients of a region's planes share: the row origin, the grid, the slots filled
+// so far (nl lower bounds from the front, nu upper bounds from the back).
+struct RowCoef {
+    float4 *E;
+    float pb0, pc0, K, inv_h, h, eps;
+    int nl, nu;
+    __device__ __forceinline__ void put(bool lower, float4 c) {
+        E[lower ? nl : KMAX - 1 - nu] = c;
+        nl += lower;
+        nu += !lower;
+    }
+    __device__ __forceinline__ float offset(float3 m, float w) const {
+        return fmaf(m.y, pb0, fmaf(m.z, pc0, w)) + eps;
+    }
+    __device__ __forceinline__ void gate(float3 m, float r0) {  // m.x == 0
+        const float s = -0x1p100f;
+        put(true, make_float4(s * r0, s * (m.y * h), s * (m.z * h), 0.f));
+    }
+    // one reciprocal and one store for either sign of m.x: the lanes of a warp hold planes of all
+    // orientations, so a branch per sign ran both sides for every plane
+    __device__ __forceinline__ void add(float3 m, float w) {
+        const float r0 = offset(m, w);
+        if (m.x == 0.f) {
+            gate(m, r0);
+        } else {
+            const float inv = 1.f / m.x;
+            put(m.x > 0.f, make_float4(fmaf(-r0 * inv, inv_h, -K), -m.y * inv, -m.z * inv, 0.f));
         }
     }
+    // the planes (m, w1) and (-m, w2) of a slab: the same slopes, one reciprocal
+    __device__ __forceinline__ void add_slab(float3 m, float w1, float w2) {
+        const float3 n = make_float3(-m.x, -m.y, -m.z);
+        const float r1 = offset(m, w1), r2 = offset(n, w2);
+        if (m.x == 0.f) {
+            gate(m, r1);
+            gate(n, r2);
+        } else {
+            const float inv = 1.f / m.x, b = -m.y * inv, c = -m.z * inv;
+            put(m.x > 0.f, make_float4(fmaf(-r1 * inv, inv_h, -K), b, c, 0.f));
+            put(m.x < 0.f, make_float4(fmaf(r2 * inv, inv_h, -K), b, c, 0.f));
+        }
+    }
+};
+
+// A queued row: feature id, and len | start along the scan axis << 6 | b << 11 | c << 16 | axis << 21
+// (tile-local).  A warp's queue: ring slot of its first row, rows and points waiting (warp-uniform).
+struct RowQueue {
+    int head, rows, points;
+};
+
+// The first 32 points of the warp's queued rows (all of them when fewer wait), one per lane:
+// distance to the row's feature, and the merge into the tile's keys (Algorithm 1).  A row that is
+// only begun keeps its rest in the queue, so that a step with points to spare runs full.
+template <int TY, int TZ, int NT>
+__device__ __forceinline__ void eval_step(const Feat &F, const GridP &g, TileSmem<TY, TZ, NT> &S, RowQueue &q, int x0,
+                                          int y0, int z0, unsigned &cand) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint2 *const Q = S.rowq[warp];
+    uint2 e = make_uint2(0u, 0u);
+    if (lane < q.rows) e = Q[(q.head + lane) & 63];
+    const int len = (int)(e.y & 63u);
+    const int pincl = warp_incl_scan(len), first = pincl - len;
+    const int n = min(q.points, 32);
+    // every row has a point, so the rows' first points are distinct: bit i of `heads` marks the row
+    // that starts at point i
+    const unsigned heads = __reduce_or_sync(FULL, len > 0 && first < 32 ? 1u << first : 0u);
+    const unsigned mine = heads & (0xffffffffu >> (31 - lane));
+    const int ro = __popc(mine) - 1;
+    const unsigned fid_o = __shfl_sync(FULL, e.x, ro), re = __shfl_sync(FULL, e.y, ro);
+    if (lane < n) {
+        const int la = (int)((re >> 6) & 31u) + (lane - (31 - __clz(mine))), lb = (int)((re >> 11) & 31u),
+                  lc = (int)((re >> 16) & 31u), ax = (int)(re >> 21);
+        const int lx = ax == 0 ? la : lb;
+        const int ly = ax == 1 ? la : (ax == 0 ? lb : lc);
+        const int lz = ax == 2 ? la : lc;
+        const int fid = (int)fid_o;
+        const int type = feat_type(F, fid), id = feat_local(F, fid, type);
+        bool neg, unc;
+        const float d = eval_any(F, g, type, id, x0 + lx, y0 + ly, z0 + lz, neg, unc);
+        if (d < g.W) {
+            atomicMin(S.key + (lz * TY + ly) * TILE_X + lx, make_key(d, fid, unc, neg));
+            cand++;
+        }
+    }
+    const int done = __popc(__ballot_sync(FULL, len > 0 && pincl <= n));  // rows with all their points evaluated
+    if (lane == done && first < n) Q[(q.head + lane) & 63].y = e.y + (unsigned)((n - first) * ((1 << 6) - 1));
+    __syncwarp();
+    q.head = (q.head + done) & 63;
+    q.rows -= done;
+    q.points -= n;
 }
 
-// Set-up of one region of a band tile (pair q of the tile's list; none when q >= qend) into slot
-// `slot` of the tile's shared arrays: its scan axis (the longest side of its box in the tile), its
-// row count (returned) and its span coefficients (Algorithm 2's half-spaces as bounds linear in a
-// row's two indices, plus the quadratic bound of a vertex ball or an edge cylinder).
-template <int TY, int TZ>
-__device__ __forceinline__ int setup_region(const Feat &F, const GridP &g, const int2 *pairs, int64_t q, int64_t qend,
-                                            int x0, int y0, int z0, TileSmem<TY, TZ> &S, int slot) {
+// Set-up of one region of a band tile (its pair; has: the thread has one) into slot `slot` of the
+// tile's shared arrays: its scan axis (the longest side of its box in the tile), its row count
+// (returned) and its span coefficients (Algorithm 2's half-spaces as bounds linear in a row's two
+// indices, plus the quadratic bound of a vertex ball or an edge cylinder).
+template <int TY, int TZ, int NT>
+__device__ __forceinline__ int setup_region(const Feat &F, const GridP &g, int2 pr, bool has, int x0, int y0, int z0,
+                                            TileSmem<TY, TZ, NT> &S, int slot) {
+    if (!has) return 0;
     const float3 org = make_float3(g.ox, g.oy, g.oz);
-    int fid = 0, lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1}, type = FACE, id = 0;
-    if (q < qend) {
-        const int2 pr = __ldg(pairs + q);
-        fid = pr.x;
-        type = feat_type(F, fid);
-        id = feat_local(F, fid, type);
-        const unsigned bx = (unsigned)pr.y;
-        lo[0] = x0 + (int)(bx & 31u); hi[0] = x0 + (int)((bx >> 5) & 31u);
-        lo[1] = y0 + (int)((bx >> 10) & 15u); hi[1] = y0 + (int)((bx >> 14) & 15u);
-        lo[2] = z0 + (int)((bx >> 18) & 15u); hi[2] = z0 + (int)((bx >> 22) & 15u);
-    }
+    const int fid = pr.x, type = feat_type(F, fid), id = feat_local(F, fid, type);
+    const unsigned box = (unsigned)pr.y;
+    const int lo[3] = {x0 + (int)(box & 31u), y0 + (int)((box >> 10) & 15u), z0 + (int)((box >> 18) & 15u)};
+    const int hi[3] = {x0 + (int)((box >> 5) & 31u), y0 + (int)((box >> 14) & 15u), z0 + (int)((box >> 22) & 15u)};
     const int n0 = hi[0] - lo[0] + 1, n1 = hi[1] - lo[1] + 1, n2 = hi[2] - lo[2] + 1;
     const int ax = (n0 >= n1 && n0 >= n2) ? 0 : (n1 >= n2 ? 1 : 2);
     const int bx = ax == 0 ? 1 : 0, cx = ax == 2 ? 1 : 2;
     const int nb = bx == 0 ? n0 : n1, nc = cx == 1 ? n1 : n2;
-    const int nrows = (n0 > 0 && n1 > 0 && n2 > 0) ? nb * nc : 0;
     const int la = ax == 0 ? lo[0] : (ax == 1 ? lo[1] : lo[2]);
     const int ha = ax == 0 ? hi[0] : (ax == 1 ? hi[1] : hi[2]);
     const int lb = bx == 0 ? lo[0] : lo[1];
     const int lc = cx == 1 ? lo[1] : lo[2];
     S.fid[slot] = fid;
-    S.ax[slot] = (unsigned char)ax;
     // tile-local starts: a row's points are (a, b, c) = (lo_a + j, lo_b + ib, lo_c + ic)
     const int loa = la - (ax == 0 ? x0 : (ax == 1 ? y0 : z0));
     const int lob = lb - (bx == 0 ? x0 : y0);
     const int loc = lc - (cx == 1 ? y0 : z0);
-    const int nbc = max(nb, 1);
-    int nl = 0, nu = 0;
     // quadratic row bound in index units: vertex (j_v, db0, dc0, R^2); edge (Qa, Qb, Qc, R^2),
     // (t_a, t_b, t_c, -) with Q the edge point a seen from the row origin; faces none (their
     // slab planes bound the distance)
-    float4 q0v = make_float4(0.f, 0.f, 0.f, 0.f), q1v = make_float4(0.f, 0.f, 0.f, Q_NONE);
-    if (nrows > 0) {
-        // whole-grid indices of the box's first row (z indices carry the slab's first layer)
-        const int la_g = la + (ax == 2 ? g.kofs : 0), lc_g = lc + (cx == 2 ? g.kofs : 0);
-        const float pb0 = fmaf((float)lb + 0.5f, g.h, comp3(org, bx));
-        const float pc0 = fmaf((float)lc_g + 0.5f, g.h, comp3(org, cx));
-        const float K = comp3(org, ax) * g.inv_h + 0.5f + (float)la_g;  // j = (p_a - o_a)/h - 1/2 - lo_a
-        float4 *E = S.coef[slot];  // written directly to shared memory
-        if (type == FACE) {
-            const float4 *r = F.face_rec + 4 * id;
-            const float4 n = __ldg(r);
-            add_coef(E, nl, nu, make_float4(n.x, n.y, n.z, n.w + g.W), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, make_float4(-n.x, -n.y, -n.z, g.W - n.w), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, __ldg(r + 1), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, __ldg(r + 2), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, __ldg(r + 3), ax, bx, cx, pb0, pc0, K, g);
-        } else if (type == EDGE) {
-            const float4 *r = F.edge_rec + 5 * id;
-            const float4 a = __ldg(r), tt = __ldg(r + 1);
-            add_coef(E, nl, nu, make_float4(tt.x, tt.y, tt.z, -tt.w), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, make_float4(-tt.x, -tt.y, -tt.z, tt.w + a.w), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, __ldg(r + 2), ax, bx, cx, pb0, pc0, K, g);
-            add_coef(E, nl, nu, __ldg(r + 3), ax, bx, cx, pb0, pc0, K, g);
-            // the wedge planes do not bound the distance to the edge line: add the cylinder
-            // |(p - a) x t| <= W (+ tolerance and a slack of 1/64 cell), which only removes
-            // points the merge would reject (d >= W)
-            const float3 av = f3(a), tv = f3(tt);
-            const float Rs = (g.W + g.eps) * g.inv_h + 1.f / 64.f;
-            q0v = make_float4((comp3(org, ax) - comp3(av, ax)) * g.inv_h + 0.5f + (float)la_g,
-                              (pb0 - comp3(av, bx)) * g.inv_h, (pc0 - comp3(av, cx)) * g.inv_h, Rs * Rs);
-            q1v = make_float4(comp3(tv, ax), comp3(tv, bx), comp3(tv, cx), Q_EDGE);
-        } else {
-            const float4 v = __ldg(F.vert_rec + 3 * id), nv = __ldg(F.vert_rec + 3 * id + 1);
-            const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), MAXVP);
-            for (int k = 0; k < cnt; k++)
-                add_coef(E, nl, nu, __ldg(F.vert_plane + s0 + k), ax, bx, cx, pb0, pc0, K, g);
-            const float3 vv = f3(v);
-            const float Rh = (g.W + g.eps) * g.inv_h;
-            q0v = make_float4((comp3(vv, ax) - comp3(org, ax)) * g.inv_h - 0.5f - (float)la_g,
-                              (pb0 - comp3(vv, bx)) * g.inv_h, (pc0 - comp3(vv, cx)) * g.inv_h, Rh * Rh);
-            q1v.w = Q_VERT;
+    float4 q0v = make_float4(0.f, 0.f, 0.f, 0.f), q1v = q0v;
+    int kind = Q_NONE;
+    // whole-grid indices of the box's first row (z indices carry the slab's first layer)
+    const int la_g = la + (ax == 2 ? g.kofs : 0), lc_g = lc + (cx == 2 ? g.kofs : 0);
+    RowCoef rc;
+    rc.E = S.coef[slot];
+    rc.pb0 = fmaf((float)lb + 0.5f, g.h, comp3(org, bx));
+    rc.pc0 = fmaf((float)lc_g + 0.5f, g.h, comp3(org, cx));
+    rc.K = comp3(org, ax) * g.inv_h + 0.5f + (float)la_g;  // j = (p_a - o_a)/h - 1/2 - lo_a
+    rc.inv_h = g.inv_h;
+    rc.h = g.h;
+    rc.eps = g.eps;
+    rc.nl = rc.nu = 0;
+    if (type == FACE) {
+        const float4 *r = F.face_rec + 4 * id;
+        const float4 n = __ldg(r), s1 = __ldg(r + 1), s2 = __ldg(r + 2), s3 = __ldg(r + 3);
+        rc.add_slab(along(n, ax), n.w + g.W, g.W - n.w);
+        rc.add(along(s1, ax), s1.w);
+        rc.add(along(s2, ax), s2.w);
+        rc.add(along(s3, ax), s3.w);
+    } else if (type == EDGE) {
+        const float4 *r = F.edge_rec + 5 * id;
+        const float4 a = __ldg(r), tt = __ldg(r + 1), p2 = __ldg(r + 2), p3 = __ldg(r + 3);
+        rc.add_slab(along(tt, ax), -tt.w, tt.w + a.w);
+        rc.add(along(p2, ax), p2.w);
+        rc.add(along(p3, ax), p3.w);
+        // the wedge planes do not bound the distance to the edge line: add the cylinder
+        // |(p - a) x t| <= W (+ tolerance and a slack of 1/64 cell), which only removes
+        // points the merge would reject (d >= W)
+        const float3 av = f3(a), tv = f3(tt);
+        const float Rs = (g.W + g.eps) * g.inv_h + 1.f / 64.f;
+        q0v = make_float4((comp3(org, ax) - comp3(av, ax)) * g.inv_h + 0.5f + (float)la_g,
+                          (rc.pb0 - comp3(av, bx)) * g.inv_h, (rc.pc0 - comp3(av, cx)) * g.inv_h, Rs * Rs);
+        q1v = make_float4(comp3(tv, ax), comp3(tv, bx), comp3(tv, cx), 0.f);
+        kind = Q_EDGE;
+    } else {
+        const float4 v = __ldg(F.vert_rec + 3 * id), nv = __ldg(F.vert_rec + 3 * id + 1);
+        const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), MAXVP);
+        for (int k = 0; k < cnt; k++) {
+            const float4 P = __ldg(F.vert_plane + s0 + k);
+            rc.add(along(P, ax), P.w);
         }
+        const float3 vv = f3(v);
+        const float Rh = (g.W + g.eps) * g.inv_h;
+        q0v = make_float4((comp3(vv, ax) - comp3(org, ax)) * g.inv_h - 0.5f - (float)la_g,
+                          (rc.pb0 - comp3(vv, bx)) * g.inv_h, (rc.pc0 - comp3(vv, cx)) * g.inv_h, Rh * Rh);
+        kind = Q_VERT;
     }
-    for (int k = nl; k < KMAX - nu; k++) S.coef[slot][k] = make_float4(1e30f, 0.f, 0.f, 0.f);
-    S.quad[slot][0] = q0v;
-    S.quad[slot][1] = q1v;
-    S.qkind[slot] = (unsigned char)q1v.w;
+    for (int k = rc.nl; k < KMAX - rc.nu; k++) rc.E[k] = make_float4(1e30f, 0.f, 0.f, 0.f);
+    if (type != FACE) {
+        S.quad[slot][0] = q0v;
+        S.quad[slot][1] = q1v;
+    }
+    S.axq[slot] = (unsigned char)(ax | kind << 2);
     // rinfo: x = nb | nl << 8 | span_hi << 12 | lo_a << 17 | lo_b << 22 | lo_c << 27 (tile-local,
     // 5 bits each), y = 1 / nb
-    S.rinfo[slot] = make_uint2((unsigned)(nbc | (nl << 8) | (max(ha - la, 0) << 12) | (loa << 17) | (lob << 22) |
+    S.rinfo[slot] = make_uint2((unsigned)(nb | (rc.nl << 8) | ((ha - la) << 12) | (loa << 17) | (lob << 22) |
                                        (loc << 27)),
-                            __float_as_uint(1.f / (float)nbc));
-    return nrows;
+                            __float_as_uint(1.f / (float)nb));
+    return nb * nc;
 }
 
 // The span of row `local` (in the region's row order) of the region in slot reg: its length (0 for
-// an empty row) and, in `packed`, its queue record slot | start along a << 8 | len << 13 |
-// b << 19 | c << 24 (tile-local).
-template <int TY, int TZ>
-__device__ __forceinline__ int row_span(const TileSmem<TY, TZ> &S, int reg, int local, int &packed) {
+// an empty row) and, in `packed`, its place in a queue record (see RowQueue).
+template <int TY, int TZ, int NT>
+__device__ __forceinline__ int row_span(const TileSmem<TY, TZ, NT> &S, int reg, int local, unsigned &packed) {
     const uint2 ri = S.rinfo[reg];
     const int nbv = (int)(ri.x & 255u), nl = (int)((ri.x >> 8) & 15u);
     const int ic = (int)(((float)local + 0.5f) * __uint_as_float(ri.y));  // exact for these sizes
@@ -723,8 +764,8 @@ __device__ __forceinline__ int row_span(const TileSmem<TY, TZ> &S, int reg, int 
         if (k < nl) lo_f = fmaxf(lo_f, v);
         else hi_f = fminf(hi_f, v);
     }
-    const int qk = S.qkind[reg];
-    if (qk == (int)Q_VERT) {  // ball around the vertex
+    const int axq = S.axq[reg], qk = axq >> 2;
+    if (qk == Q_VERT) {  // ball around the vertex
         const float4 bl = S.quad[reg][0];
         const float db = bl.y + fb, dc = bl.z + fc;
         const float q2 = bl.w - db * db - dc * dc;
@@ -735,7 +776,7 @@ __device__ __forceinline__ int row_span(const TileSmem<TY, TZ> &S, int reg, int 
             lo_f = fmaxf(lo_f, bl.x - sq);
             hi_f = fminf(hi_f, bl.x + sq);
         }
-    } else if (qk == (int)Q_EDGE && hi_f - lo_f > 2.f) {
+    } else if (qk == Q_EDGE && hi_f - lo_f > 2.f) {
         // cylinder around the edge line, c2 j^2 + c1 j + c0 <= 0: only for spans of more than
         // a few points (long spans come from wide wedges, whose planes leave the radius open)
         const float4 cq = S.quad[reg][0], q1 = S.quad[reg][1];
@@ -767,85 +808,117 @@ __device__ __forceinline__ int row_span(const TileSmem<TY, TZ> &S, int reg, int 
     const float fz = fmaxf(fminf(hi_f + sl, span_hi), -1.f);
     const int ja = (int)ceilf(fa), jb = (int)floorf(fz);
     const int len = open ? max(jb - ja + 1, 0) : 0;
-    packed = reg | ((int)((ri.x >> 17) & 31u) + ja) << 8 | (len << 13) |
-             (((int)((ri.x >> 22) & 31u) + ib) << 19) | (((int)(ri.x >> 27) + ic) << 24);
+    packed = (unsigned)(len | ((int)((ri.x >> 17) & 31u) + ja) << 6 | ((int)((ri.x >> 22) & 31u) + ib) << 11 |
+                        ((int)(ri.x >> 27) + ic) << 16 | (axq & 3) << 21);
     return len;
 }
 
-// Queue a row (len > 0) in the warp's ring; once 32 rows wait, evaluate their points.
-template <int TY, int TZ>
-__device__ __forceinline__ void queue_row(const Feat &F, const GridP &g, TileSmem<TY, TZ> &S, int len, int packed,
-                                          int &qh, int &qn, int x0, int y0, int z0, unsigned &cand) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned hit = __ballot_sync(FULL, len > 0);
-    if (len > 0) S.rowq[warp][(qh + qn + __popc(hit & ((1u << lane) - 1u))) & 63] = (unsigned)packed;
-    qn += __popc(hit);
-    __syncwarp();
-    if (qn >= 32) {
-        eval_rows<TY, TZ>(F, g, S, S.rowq[warp], qh, 32, x0, y0, z0, cand);
-        qh = (qh + 32) & 63;
-        qn -= 32;
-    }
-}
-// the rest of the warp's queue
-template <int TY, int TZ>
-__device__ __forceinline__ void flush_rows(const Feat &F, const GridP &g, TileSmem<TY, TZ> &S, int &qh, int &qn,
-                                           int x0, int y0, int z0, unsigned &cand) {
-    const int warp = threadIdx.x >> 5;
-    while (qn > 0) {
-        const int m = min(qn, 32);
-        eval_rows<TY, TZ>(F, g, S, S.rowq[warp], qh, m, x0, y0, z0, cand);
-        qh = (qh + m) & 63;
-        qn -= m;
-    }
-}
-
-// All regions of one band tile.  Per region: its box in the tile (packed in the pair by the
-// binning), its scan axis, its row count and its span coefficients (setup_region); per row: the
-// span (row_span, Algorithm 2 on a grid line); non-empty rows wait in a per-warp queue until 32
-// are ready, then their points are flattened over the lanes, evaluated and merged into the tile's
-// keys with a shared-memory atomicMin (Algorithm 1, eval_rows).  The warps take equal chunks of
-// at most 32 regions (a multiple of the warp count of them, so that a tile with few regions still
-// uses every warp) from a shared counter and work on them without block barriers: one lane per
-// region sets it up, a warp scan numbers the chunk's rows, and each lane takes one row, found by a
-// shuffle search of the scan.  (Handing out a tile's rows block-wide in batches of 32 was measured
-// slower on the knot tube and no faster on the torus.)
-template <int TY, int TZ>
+// All regions of one band tile, q0 .. q3 - 1 of the pair list.  Per region: its box in the tile
+// (packed in the pair by the binning), its scan axis, its row count and its span coefficients
+// (setup_region, one lane each); per row: the span (row_span, Algorithm 2 on a grid line, one lane
+// each); non-empty rows wait in a per-warp queue until 32 points are ready, which are evaluated and
+// merged into the tile's keys with a shared-memory atomicMin (Algorithm 1, eval_step).
+//
+// The set-up's cost is per warp whatever the number of lanes with a region (about 530 instructions, a
+// third of the kernel's on the knot tube).  So a tile of at most NT regions is set up by as few
+// warps as hold them, one pass for the whole CTA, and the warps then take its rows in batches of
+// 32 from a shared counter (a fixed share of the rows per warp left the warps with the face rows, which
+// hold nearly all points, to finish alone: 293 us on the 200 k-triangle sphere at 512^3 against 210).
+// A larger tile is worked on without block barriers: the warps take equal chunks of at most 32
+// regions from a shared counter, each with its own rows, the next chunk's pairs on their way meanwhile.
+// With equal chunks for every tile, rows queued by the 32 with what was left of them evaluated at the
+// end of each chunk, and a branch per plane orientation in the set-up, the kernel took 689 us on the
+// knot tube at 512^3, 1593 us at 1024^3, 362 + 76 us on the batch of 24; now 641, 1430, 283 + 79 us.
+template <int TY, int TZ, int NT>
 __device__ void process_band_tile(const Feat &F, const GridP &g, const int2 *pairs, int64_t q0, int64_t q3,
-                                  int x0, int y0, int z0, TileSmem<TY, TZ> &S, unsigned &cand, unsigned &rows,
+                                  int x0, int y0, int z0, TileSmem<TY, TZ, NT> &S, unsigned &cand, unsigned &rows,
                                   unsigned &hits) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = threadIdx.x;
-    const int64_t npairs = q3 - q0;
-    if (npairs <= 0) return;  // (after a pair-list overflow a band tile may have no stored pairs)
-    int qh = 0, qn = 0;       // head and length of this warp's row queue
-    const int64_t nchunks = (NT / 32) * ((npairs + NT - 1) / NT);  // >= NT / 32
-    const int cs = (int)((npairs + nchunks - 1) / nchunks);          // >= 1: every chunk advances
-    for (;;) {
-        int chunk = 0;  // this warp's next chunk of the tile's regions
-        if (lane == 0) chunk = atomicAdd(&S.next, 1);
-        chunk = __shfl_sync(FULL, chunk, 0);
-        const int64_t base = q0 + (int64_t)cs * chunk;
-        if (base >= q3) break;
-        const int nrows = setup_region<TY, TZ>(F, g, pairs, base + lane, min(base + cs, q3), x0, y0, z0, S, t);
-        // rows of the warp's regions, numbered by a warp scan
+    const int npairs = (int)(q3 - q0);  // (0 after a pair-list overflow: the tile has no stored pairs)
+    const bool one_pass = npairs <= NT;
+    // chunks: a multiple of the warp count, so that every warp has a share
+    const int nchunks = (NT / 32) * ((npairs + NT - 1) / NT);
+    const int cs = one_pass ? 32 : (npairs + nchunks - 1) / nchunks;
+    int base = cs * warp;  // this warp's regions: base .. base + cs - 1 of the tile's
+    bool has = lane < cs && base + lane < npairs;
+    int2 pr = has ? __ldg(pairs + q0 + base + lane) : make_int2(0, 0);
+    for (int e = t; e < TILE_X * TY * TZ; e += NT) S.key[e] = ~0ull;
+    if (t == 0) S.next = one_pass ? 0 : NT / 32;  // batches of rows, or chunks of regions
+    RowQueue q = {0, 0, 0};
+    __syncthreads();
+    while (base < npairs || one_pass) {
+        int chunk = 0;
+        if (!one_pass && lane == 0) chunk = atomicAdd(&S.next, 1);
+        const int nrows = setup_region<TY, TZ, NT>(F, g, pr, has, x0, y0, z0, S, t);
+        // number the rows: pre[i] is the first row of region i (of the pass, or of the warp's chunk)
         const int incl = warp_incl_scan(nrows);
-        const int R = __shfl_sync(FULL, incl, 31);
-        __syncwarp();
-        for (int rbase = 0; rbase < R; rbase += 32) {
-            const int r = rbase + lane;
-            const int own = min(warp_owner(incl, r), 31);  // lane whose region holds row r
-            const int r0 = __shfl_sync(FULL, incl - nrows, own);
-            int len = 0, packed = 0;
-            if (r < R) {
-                len = row_span<TY, TZ>(S, warp * 32 + own, r - r0, packed);
+        unsigned short *pre = S.pre;  // (at most NT - 1 regions of at most 16 x 8 rows come before one)
+        int nreg = npairs, r = 0, r_end, own = 0;  // regions, this warp's rows, the region holding row r
+        if (one_pass) {
+            if (lane == 31) S.wsum[warp] = incl;
+            __syncthreads();
+            int before = 0, total = 0;
+#pragma unroll
+            for (int w = 0; w < NT / 32; w++) {
+                const int c = S.wsum[w];
+                before += w < warp ? c : 0;
+                total += c;
+            }
+            pre[t] = (unsigned short)(before + incl - nrows);
+            __syncthreads();
+            r_end = total;
+        } else {
+            chunk = __shfl_sync(FULL, chunk, 0);
+            pre += warp * 33;
+            pre[lane] = (unsigned short)(incl - nrows);
+            nreg = min(cs, npairs - base);
+            r_end = __shfl_sync(FULL, incl, 31);
+            base = cs * chunk;
+            has = lane < cs && base + lane < npairs;
+            if (has) pr = __ldg(pairs + q0 + base + lane);
+            __syncwarp();
+        }
+        const int slot0 = one_pass ? 0 : warp * 32;
+        for (;; r += 32) {
+            if (one_pass) {  // the next batch of 32 rows from the shared counter, and the region it starts in
+                int b = 0;
+                if (lane == 0) b = atomicAdd(&S.next, 1);
+                r = 32 * __shfl_sync(FULL, b, 0);
+                if (r >= r_end) break;
+                const int c = lane * (NT / 32);
+                own = (__popc(__ballot_sync(FULL, c < nreg && pre[c] <= r)) - 1) * (NT / 32);
+                const int d = own + lane;
+                own += __popc(__ballot_sync(FULL, lane < NT / 32 && d < nreg && pre[d] <= r)) - 1;
+            } else if (r >= r_end) {
+                break;
+            }
+            // every region has a row, so the next 32 regions' first rows are distinct: bit i of
+            // `heads` marks the region that starts at row r + i
+            const int nx = own + 1 + lane;
+            const int first = nx < nreg ? pre[nx] - r : 64;
+            const unsigned heads = __reduce_or_sync(FULL, first < 32 ? 1u << first : 0u);
+            const int reg = own + __popc(heads & (0xffffffffu >> (31 - lane)));
+            own += __popc(__ballot_sync(FULL, first <= 32));
+            int len = 0;
+            unsigned packed = 0;
+            if (r + lane < r_end) {
+                len = row_span<TY, TZ, NT>(S, slot0 + reg, r + lane - pre[reg], packed);
                 rows++;
                 hits += len > 0;
             }
-            queue_row<TY, TZ>(F, g, S, len, packed, qh, qn, x0, y0, z0, cand);
+            const unsigned hit = __ballot_sync(FULL, len > 0);
+            if (len > 0)
+                S.rowq[warp][(q.head + q.rows + __popc(hit & ((1u << lane) - 1u))) & 63] =
+                    make_uint2((unsigned)S.fid[slot0 + reg], packed);
+            q.rows += __popc(hit);
+            q.points += __reduce_add_sync(FULL, len);
+            __syncwarp();
+            while (q.points >= 32) eval_step<TY, TZ, NT>(F, g, S, q, x0, y0, z0, cand);
         }
-        flush_rows<TY, TZ>(F, g, S, qh, qn, x0, y0, z0, cand);  // region slots are rewritten by the next chunk
-        __syncwarp();
+        if (one_pass) break;
+        __syncwarp();  // the region slots are rewritten by the next chunk
     }
+    while (q.points > 0) eval_step<TY, TZ, NT>(F, g, S, q, x0, y0, z0, cand);
 }
 
 // decode one merged key into the output value / winner, queueing FP64 re-decisions; entry tells
@@ -885,8 +958,8 @@ __device__ __forceinline__ float decode_key(unsigned long long key, const GridP 
 // takes consecutive slots for its entries with one atomicAdd (no block barrier, so the atomic's
 // latency overlaps the other warps' work) and its threads write their entries, re-reading the
 // winners from the tile's keys, which stay in shared memory until the tile's end.
-template <int TY, int TZ>
-__device__ __forceinline__ void list_write(const Prob &pr, const TileSmem<TY, TZ> &S, unsigned emask, int x0, int y0,
+template <int TY, int TZ, int NT>
+__device__ __forceinline__ void list_write(const Prob &pr, const TileSmem<TY, TZ, NT> &S, unsigned emask, int x0, int y0,
                                            int z0, bool vec_rows, bool &overflow) {
     const int lane = threadIdx.x & 31;
     const unsigned c = __popc(emask);
@@ -959,21 +1032,23 @@ __global__ void k_band_flags(const uint32_t *bin_start, int64_t n_tiles, uint32_
 constexpr int FILL_CHUNK = 32;
 
 //
-// A band tile with more than SPLIT_MIN pairs (a densely subdivided part of a mesh puts tens of
-// thousands of regions into a few tiles) is split: while slots last (split_cap), it takes a slot
-// and becomes S = min(ceil(np / SPLIT_PAIRS), SPLIT_MAX_ITEMS) work items, each a contiguous part
-// of its pairs, listed in split_items for the SPLIT launch of the tile kernel; its own entry in
-// band_list becomes -1 (skipped).  An item packs (tile, slot | item << 12 | S << 20).  Tiles of a
-// few thousand pairs (the knot tube at 512^3 has some) stay whole: their split items, run in a
-// launch of their own, cost more than they gain.
-constexpr int SPLIT_MIN = 8192, SPLIT_PAIRS = 2048, SPLIT_MAX_ITEMS = 64, SPLIT_SLOTS = 256;
+// A band tile with many pairs (a densely subdivided part of a mesh puts tens of thousands of regions
+// into a few tiles) is split: while slots last (split_cap), it takes a slot and becomes
+// S = min(ceil(np / SPLIT_PAIRS), SPLIT_MAX_ITEMS) work items, each a contiguous part of its pairs,
+// listed in split_items for the SPLIT launch of the tile kernel; its own entry in band_list becomes
+// -1 (skipped).  An item packs (tile, slot | item << 12 | S << 20).  Many is more than the mean work of
+// a CTA of the launch, within [SPLIT_MIN, SPLIT_MAX]: such a tile would be finished last.  On the
+// batch of 24 uneven meshes that took the two launches from 69 + 345 us (with 8192 always) to
+// 79 + 283; the knot tube at 512^3, whose tiles of up to 6,000 pairs are no more than a CTA's mean work,
+// loses 90 us when they are split (the items' launch comes first) and keeps them whole.
+constexpr int SPLIT_MIN = 2048, SPLIT_MAX = 8192, SPLIT_PAIRS = 1024, SPLIT_MAX_ITEMS = 64, SPLIT_SLOTS = 256;
 // the launch clears tile_hist, tile_cursor, n_split and n_split_items with one memset
 static_assert(offsetof(DevCounters, n_split_items) == offsetof(DevCounters, tile_hist) + 33 * sizeof(unsigned),
               "the per-launch tile-list counters must be contiguous");
 
 __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const uint32_t *band_pos,
                              int32_t *band_list, int32_t *empty_list, DevCounters *ctr, int lpt, int2 *split_items,
-                             int split_cap) {
+                             int split_cap, int n_ctas) {
     dep_wait();
     dep_next();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -984,7 +1059,8 @@ __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const u
         return;
     }
     int32_t entry = (int32_t)t;
-    if (np > (uint32_t)SPLIT_MIN && split_cap > 0) {
+    const uint32_t split_from = min(max(bin_start[3 * n_tiles] / (uint32_t)n_ctas, (uint32_t)SPLIT_MIN), (uint32_t)SPLIT_MAX);
+    if (np > split_from && split_cap > 0) {
         const unsigned slot = atomicAdd(&ctr->n_split, 1u);
         if (slot < (unsigned)split_cap) {
             const int S = (int)min((np + SPLIT_PAIRS - 1) / SPLIT_PAIRS, (uint32_t)SPLIT_MAX_ITEMS);
@@ -1008,7 +1084,7 @@ __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const u
 // single-problem call, and most chunks of a batch, belong to one), so a whole tile costs its index
 // arithmetic and, per thread, TY * TZ / 32 coalesced 16-byte stores; tiles cut by the grid's edge
 // or rows not 16-byte aligned take the per-point path.
-template <int TY, int TZ>
+template <int TY, int TZ, int NT>
 __device__ __forceinline__ void fill_chunk(const Prob *P, const long long *tile_base, int n, const int32_t *empty_list,
                                            int64_t e0, int64_t e1) {
     long long tb_lo = 1, tb_hi = 0;  // tile range of the loaded problem (empty: load on first use)
@@ -1063,7 +1139,7 @@ __device__ __forceinline__ void fill_chunk(const Prob *P, const long long *tile_
 // back into shared memory (and clears the slot for the next launch) and returns true: it decodes
 // the tile.  No CTA waits for another.  Kept out of line, so that the band work of the tile kernel
 // compiles as without it (inlined, it cost the kernel about 12 %).
-template <int TP>
+template <int TP, int NT>
 __device__ __noinline__ bool split_merge(const Outputs &o, unsigned long long *key, int slot, int n_items, int &s_last) {
     unsigned long long *gk = o.split_keys + (size_t)slot * TP;
     for (int e = threadIdx.x; e < TP; e += NT) {
@@ -1096,8 +1172,8 @@ __device__ __noinline__ bool split_merge(const Outputs &o, unsigned long long *k
 // plain kernel carries none of its code).  SPLIT: the launch that works on the items of split
 // tiles (k_tile_lists) alone, before the launch of the band tiles and the fill; compiled apart
 // too, since the split path in the same kernel cost the band work about 12 %.
-template <int TY, int TZ, bool LIST, bool SPLIT>
-__global__ void __launch_bounds__(NT, 4) k_tile(const Prob *P, const long long *tile_base, int n, Outputs o,
+template <int TY, int TZ, bool LIST, bool SPLIT, int NT>
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, const long long *tile_base, int n, Outputs o,
                                                 int64_t n_tiles, const int32_t *band_list,
                                                 const int32_t *empty_list, const uint32_t *n_band_ptr,
                                                 unsigned long long *ticket, int dense) {
@@ -1105,7 +1181,7 @@ __global__ void __launch_bounds__(NT, 4) k_tile(const Prob *P, const long long *
     dep_next();
     constexpr int TP = TILE_X * TY * TZ;
     extern __shared__ __align__(16) unsigned char tile_smem[];
-    TileSmem<TY, TZ> &S = *reinterpret_cast<TileSmem<TY, TZ> *>(tile_smem);
+    TileSmem<TY, TZ, NT> &S = *reinterpret_cast<TileSmem<TY, TZ, NT> *>(tile_smem);
     __shared__ unsigned s_cand, s_band, s_ovf, s_rows, s_hits, s_pairs;
     __shared__ int s_kind, s_last;
     if (threadIdx.x == 0) { s_cand = 0; s_band = 0; s_ovf = 0; s_rows = 0; s_hits = 0; s_pairs = 0; }
@@ -1147,7 +1223,7 @@ __global__ void __launch_bounds__(NT, 4) k_tile(const Prob *P, const long long *
         __syncthreads();
         if (w < 0) break;
         if (kind) {  // a chunk of empty tiles
-            fill_chunk<TY, TZ>(P, tile_base, n, empty_list, w * FILL_CHUNK, min((w + 1) * FILL_CHUNK, n_empty));
+            fill_chunk<TY, TZ, NT>(P, tile_base, n, empty_list, w * FILL_CHUNK, min((w + 1) * FILL_CHUNK, n_empty));
             continue;
         }
         {  // a band tile, or an item of a split tile
@@ -1183,13 +1259,10 @@ __global__ void __launch_bounds__(NT, 4) k_tile(const Prob *P, const long long *
                     q0 = qa;
                     q3 = qb;
                 }
-                for (int e = threadIdx.x; e < TP; e += NT) S.key[e] = ~0ull;
-                if (threadIdx.x == 0) S.next = 0;
-                __syncthreads();
-                process_band_tile<TY, TZ>(pr.F, g, o.pairs, q0, q3, x0, y0, z0, S, cand, rows, hits);
+                process_band_tile<TY, TZ, NT>(pr.F, g, o.pairs, q0, q3, x0, y0, z0, S, cand, rows, hits);
                 __syncthreads();  // every merge is in before the decode
                 if (threadIdx.x == 0) pairs += (unsigned)(q3 - q0);
-                if (SPLIT && !split_merge<TP>(o, S.key, split_slot, split_n, s_last)) continue;
+                if (SPLIT && !split_merge<TP, NT>(o, S.key, split_slot, split_n, s_last)) continue;
             }
             const bool list = LIST && is_band && pr.list != nullptr;
             const bool vec_rows = pr.vec && cx1 == x0 + TILE_X - 1;
@@ -1233,7 +1306,7 @@ __global__ void __launch_bounds__(NT, 4) k_tile(const Prob *P, const long long *
                     if (winner) __stcs(winner + idx, wid);
                 }
             }
-            if (list) list_write<TY, TZ>(pr, S, emask, x0, y0, z0, vec_rows, list_ovf);
+            if (list) list_write<TY, TZ, NT>(pr, S, emask, x0, y0, z0, vec_rows, list_ovf);
             if (is_band) __syncthreads();  // keys are reused by the next band tile
         }
     }
@@ -2117,12 +2190,12 @@ static int num_sms() {
     return n;
 }
 
-template <int TY, int TZ, bool LIST, bool SPLIT = false> static int tile_blocks_per_sm() {
+template <int TY, int TZ, bool LIST, bool SPLIT, int NT> static int tile_blocks_per_sm() {
     static int b = 0;
     if (!b) {
-        cudaFuncSetAttribute(k_tile<TY, TZ, LIST, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(TileSmem<TY, TZ>));
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tile<TY, TZ, LIST, SPLIT>, NT, sizeof(TileSmem<TY, TZ>));
+        const size_t smem = sizeof(TileSmem<TY, TZ, NT>);
+        cudaFuncSetAttribute(k_tile<TY, TZ, LIST, SPLIT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tile<TY, TZ, LIST, SPLIT, NT>, NT, smem);
         if (b <= 0) b = 1;
     }
     return b;
@@ -2552,6 +2625,35 @@ static Scratch plan_scratch(const Plan &pl) {
     return sc;
 }
 
+// The threads of a tile CTA.  With 128, six tiles are worked on at a time on an SM instead of four, each
+// with its own barriers, and a tile ends in half as many part-filled steps: the knot tube's tile
+// kernel takes 1.43 ms at 1024^3 (1.57 with 256 threads), a torus forward at 512^3 268 us (283).  On a
+// small grid, where the CTAs get few tiles each, a tile's own time counts and 256 threads are faster:
+// 77 us for a fine box at 64^3 (88 with 128), a fine torus 181 us at 128^3 (235) and 260 us at 256^3
+// (302).  The two meet at about 320^3, 16,000 tiles.
+constexpr int64_t SMALL_TILES = 16384;
+
+// the tile kernel: the items of split tiles, then the band tiles and the fill
+template <int TY, int TZ, bool LIST, int NT>
+static cudaError_t launch_tiles(int n, const Outputs &o, int64_t n_tiles, const Scratch &sc, cudaStream_t s) {
+    const size_t smem = sizeof(TileSmem<TY, TZ, NT>);
+    const uint32_t *n_band = sc.band_pos + n_tiles;
+    const int dense = sc.any_dense ? 1 : 0;
+    if (sc.split_items) {  // none in most launches: the CTAs then return at once
+        // a few tiles' items at most, and a cheap launch when there are none
+        tile_blocks_per_sm<TY, TZ, LIST, true, NT>();  // (sets the kernel's shared-memory limit once)
+        const int64_t ctas = std::min<int64_t>(n_tiles, (256 / NT) * (int64_t)num_sms());
+        const cudaError_t e = launch_dep(k_tile<TY, TZ, LIST, true, NT>, dim3((unsigned)ctas), dim3(NT), smem, s,
+                                         sc.probs, sc.tbase, n, o, n_tiles, (const int32_t *)sc.band_list,
+                                         (const int32_t *)sc.empty_list, n_band, sc.ticket, dense);
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t ctas = std::min<int64_t>(n_tiles, (int64_t)tile_blocks_per_sm<TY, TZ, LIST, false, NT>() * num_sms());
+    return launch_dep(k_tile<TY, TZ, LIST, false, NT>, dim3((unsigned)ctas), dim3(NT), smem, s, sc.probs, sc.tbase, n,
+                      o, n_tiles, (const int32_t *)sc.band_list, (const int32_t *)sc.empty_list, n_band, sc.ticket,
+                      dense);
+}
+
 // the whole pipeline of one batch: kernels and memsets only (no allocation, no synchronisation)
 template <int TY, int TZ>
 static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &sc, cudaStream_t s,
@@ -2576,7 +2678,7 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
     SDF_TRY(scan_exclusive_u32(flags, sc.band_pos, n_tiles, true, sc.scan_tmp, s, &sc.ctr->nb_status));
     SDF_TRY(launch_dep(k_tile_lists, dim3(nblk(n_tiles, 256)), dim3(256), 0, s, (const uint32_t *)sc.start, n_tiles,
                        (const uint32_t *)sc.band_pos, sc.band_list, sc.empty_list, sc.ctr, lpt, sc.split_items,
-                       sc.split_items ? SPLIT_SLOTS : 0));
+                       sc.split_items ? SPLIT_SLOTS : 0, 4 * num_sms()));
     Outputs o;
     o.pairs = sc.pairs;
     o.bin_start = sc.start;
@@ -2588,35 +2690,12 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
     o.split_keys = sc.split_keys;
     o.split_done = sc.split_done;
     if (ev) SDF_TRY(record_event(ev[1], s));
-    if (sc.any_list) {
-        const int64_t ctas = std::min<int64_t>(n_tiles, (int64_t)tile_blocks_per_sm<TY, TZ, true>() * num_sms());
-        if (sc.split_items) {  // the items of split tiles (none in most launches: the CTAs then return at once)
-            // one CTA per SM: a few tiles' items at most, and a cheap launch when there are none
-            tile_blocks_per_sm<TY, TZ, true, true>();  // (sets the kernel's shared-memory limit once)
-            const int64_t sctas = std::min<int64_t>(n_tiles, (int64_t)num_sms());
-            SDF_TRY(launch_dep(k_tile<TY, TZ, true, true>, dim3((unsigned)sctas), dim3(NT),
-                               sizeof(TileSmem<TY, TZ>), s, sc.probs, sc.tbase, n, o, n_tiles,
-                               (const int32_t *)sc.band_list, (const int32_t *)sc.empty_list,
-                               sc.band_pos + n_tiles, sc.ticket, sc.any_dense ? 1 : 0));
-        }
-        SDF_TRY(launch_dep(k_tile<TY, TZ, true, false>, dim3((unsigned)ctas), dim3(NT), sizeof(TileSmem<TY, TZ>), s,
-                           sc.probs, sc.tbase, n, o, n_tiles, (const int32_t *)sc.band_list,
-                           (const int32_t *)sc.empty_list, sc.band_pos + n_tiles, sc.ticket, sc.any_dense ? 1 : 0));
-    } else {
-        const int64_t ctas = std::min<int64_t>(n_tiles, (int64_t)tile_blocks_per_sm<TY, TZ, false>() * num_sms());
-        if (sc.split_items) {
-            // one CTA per SM: a few tiles' items at most, and a cheap launch when there are none
-            tile_blocks_per_sm<TY, TZ, false, true>();  // (sets the kernel's shared-memory limit once)
-            const int64_t sctas = std::min<int64_t>(n_tiles, (int64_t)num_sms());
-            SDF_TRY(launch_dep(k_tile<TY, TZ, false, true>, dim3((unsigned)sctas), dim3(NT),
-                               sizeof(TileSmem<TY, TZ>), s, sc.probs, sc.tbase, n, o, n_tiles,
-                               (const int32_t *)sc.band_list, (const int32_t *)sc.empty_list,
-                               sc.band_pos + n_tiles, sc.ticket, sc.any_dense ? 1 : 0));
-        }
-        SDF_TRY(launch_dep(k_tile<TY, TZ, false, false>, dim3((unsigned)ctas), dim3(NT), sizeof(TileSmem<TY, TZ>), s,
-                           sc.probs, sc.tbase, n, o, n_tiles, (const int32_t *)sc.band_list,
-                           (const int32_t *)sc.empty_list, sc.band_pos + n_tiles, sc.ticket, sc.any_dense ? 1 : 0));
-    }
+    if (n_tiles <= SMALL_TILES)
+        SDF_TRY(sc.any_list ? (launch_tiles<TY, TZ, true, 256>(n, o, n_tiles, sc, s))
+                            : (launch_tiles<TY, TZ, false, 256>(n, o, n_tiles, sc, s)));
+    else
+        SDF_TRY(sc.any_list ? (launch_tiles<TY, TZ, true, 128>(n, o, n_tiles, sc, s))
+                            : (launch_tiles<TY, TZ, false, 128>(n, o, n_tiles, sc, s)));
     if (ev) SDF_TRY(record_event(ev[2], s));
     SDF_TRY(launch_dep(k_patch<TY, TZ>, dim3(patch_blocks<TY, TZ>()), dim3(PATCH_NT), 0, s, sc.probs, sc.tbase, o));
     if (sc.fprobs)
