@@ -11,7 +11,7 @@
 //       of the point next to it in a neighbouring row (y or z), whichever row that is;
 //   (3) a grid without any band point is taken as outside.
 // Kernels: k_fill_rows applies (1) and records per row the sign at x = 0 (0 for a row without band
-// points); k_fill_lines resolves (2) by nearest-known propagation along y, then along z;
+// points); k_fill_lines_y and _z resolve (2) by nearest-known propagation along y, then along z;
 // k_fill_empty writes the rows of (2) that lie inside.  Points start at +inf (written by the tile
 // kernel), so only inside points are written.
 #include <math.h>
@@ -36,95 +36,196 @@ __device__ __forceinline__ int find_row_prob(const long long *rbase, int n, long
 // negative in the sense of the field: d < 0, or -0
 __device__ __forceinline__ bool is_neg(float v) { return signbit(v); }
 
-// One warp per x-row.  rowsign[r] = sign at x = 0 (+1 / -1), or 0 if the row has no band point.
-__global__ void k_fill_rows(const FillProb *P, const long long *rbase, int n, long long r_tot, int8_t *rowsign) {
+// What is known along a stretch of at most 32 x 32 entries, for the warp that holds it: lane c has the
+// known entries of chunk c (known: a bit each) and which of them are negative.  `carry` is the sign of
+// the last known entry before the stretch (+-1, or 0: none yet); on return the sign after it.  Lane c
+// gets the sign that holds before the first known entry of its chunk, the one of the first known
+// entry of the stretch where nothing is known before.  0 everywhere when nothing is known at all.
+__device__ __forceinline__ int chunk_signs(unsigned known, unsigned neg, int &carry) {
+    const int lane = threadIdx.x & 31;
+    const unsigned any = __ballot_sync(FULL_MASK, known != 0);
+    if (!any) return carry;
+    const int fc = __ffs(any) - 1, lc = 31 - __clz(any);
+    const unsigned fk = __shfl_sync(FULL_MASK, known, fc), fn = __shfl_sync(FULL_MASK, neg, fc);
+    const unsigned lk = __shfl_sync(FULL_MASK, known, lc), ln = __shfl_sync(FULL_MASK, neg, lc);
+    const int lead = carry ? carry : (((fn >> (__ffs(fk) - 1)) & 1u) ? -1 : 1);
+    const unsigned before = any & ((1u << lane) - 1u);
+    const int src = before ? 31 - __clz(before) : 0;
+    const unsigned sk = __shfl_sync(FULL_MASK, known, src), sn = __shfl_sync(FULL_MASK, neg, src);
+    carry = ((ln >> (31 - __clz(lk))) & 1u) ? -1 : 1;
+    return before ? (((sn >> (31 - __clz(sk))) & 1u) ? -1 : 1) : lead;
+}
+// the sign at this lane's entry of a chunk: of the nearest known entry up to it, else `in`
+__device__ __forceinline__ int sign_at(unsigned known, unsigned neg, int in) {
+    const unsigned left = known & (0xffffffffu >> (31 - (threadIdx.x & 31)));
+    return left ? (((neg >> (31 - __clz(left))) & 1u) ? -1 : 1) : in;
+}
+
+// One warp per x-row, 1024 points of it at a time.  rowsign[r] = sign at x = 0 (+1 / -1), or 0 if the
+// row has no band point.  Bound by the read of the field (4 B per point, once, eight loads in flight
+// per lane); what the points are stays in two bit masks per lane, from which the inside points are
+// written.  Reading the row up to its first band point and then again from the start, one load at a
+// time, took 63 us on a 333 x 331 x 257 grid; now 37 us.
+__global__ void __launch_bounds__(256) k_fill_rows(const FillProb *P, const long long *rbase, int n, long long r_tot,
+                                                   int8_t *rowsign) {
+    dep_wait();
+    dep_next();
     const int lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < r_tot; r += warps) {
         const int p = find_row_prob(rbase, n, r);
         const FillProb pr = P[p];
         float *row = pr.dist + (r - rbase[p]) * (long long)pr.nx;
-        // sign of the first band point of the row
-        int first = 0;  // 0: none yet, +1 / -1
-        for (int x0 = 0; x0 < pr.nx && first == 0; x0 += 32) {
-            const int x = x0 + lane;
-            const float v = x < pr.nx ? row[x] : INFINITY;
-            const bool band = isfinite(v);
-            const unsigned bm = __ballot_sync(FULL_MASK, band), nm = __ballot_sync(FULL_MASK, band && is_neg(v));
-            if (bm) {
-                const int l = __ffs(bm) - 1;
-                first = ((nm >> l) & 1u) ? -1 : 1;
+        int first = 0, carry = 0;
+        for (int s0 = 0; s0 < pr.nx; s0 += 1024) {
+            const int chunks = min(32, (pr.nx - s0 + 31) >> 5);
+            unsigned known = 0, neg = 0;
+            for (int c0 = 0; c0 < chunks; c0 += 8) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    const int x = s0 + (c0 + u) * 32 + lane;
+                    v[u] = x < pr.nx ? row[x] : INFINITY;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    const bool band = isfinite(v[u]);
+                    const unsigned bm = __ballot_sync(FULL_MASK, band), nm = __ballot_sync(FULL_MASK, band && is_neg(v[u]));
+                    if (lane == c0 + u) {
+                        known = bm;
+                        neg = nm;
+                    }
+                }
+            }
+            const int had = carry;
+            const int in = chunk_signs(known, neg, carry);
+            if (had == 0 && carry != 0) {  // the first band point of the row: it decides all before it
+                first = __shfl_sync(FULL_MASK, in, 0);
+                if (first < 0)
+                    for (int x = lane; x < s0; x += 32) row[x] = -INFINITY;
+            }
+            // the chunks that can hold inside points
+            for (unsigned todo = __ballot_sync(FULL_MASK, lane < chunks && (in < 0 || neg != 0)); todo; todo &= todo - 1) {
+                const int c = __ffs(todo) - 1;
+                const unsigned ck = __shfl_sync(FULL_MASK, known, c), cn = __shfl_sync(FULL_MASK, neg, c);
+                const int s = sign_at(ck, cn, __shfl_sync(FULL_MASK, in, c));
+                const int x = s0 + c * 32 + lane;
+                if (x < pr.nx && !((ck >> lane) & 1u) && s < 0) row[x] = -INFINITY;
             }
         }
-        if (lane == 0) rowsign[r] = (int8_t)first;
-        if (first == 0) continue;  // row without band points: resolved by the line passes
-        int carry = first;         // sign of the nearest band point to the left (or the first one)
-        for (int x0 = 0; x0 < pr.nx; x0 += 32) {
-            const int x = x0 + lane;
-            const float v = x < pr.nx ? row[x] : INFINITY;
-            const bool band = isfinite(v);
-            const unsigned bm = __ballot_sync(FULL_MASK, band), nm = __ballot_sync(FULL_MASK, band && is_neg(v));
-            if (!band && x < pr.nx) {
-                const unsigned left = bm & (0xffffffffu >> (31 - lane));  // band lanes <= this one
-                const int s = left ? (((nm >> (31 - __clz(left))) & 1u) ? -1 : 1) : carry;
-                if (s < 0) row[x] = -INFINITY;
+        if (lane == 0) rowsign[r] = (int8_t)first;  // 0: resolved by the line passes
+    }
+}
+
+// Nearest-known propagation of the row signs along y for every (problem, z), one warp per line: rows
+// without band points (0) take the sign of the nearest row before them that has some, else after them.
+// Resolved rows are marked +-2 so that k_fill_empty can tell them from rows with band points.
+__global__ void __launch_bounds__(256) k_fill_lines_y(const FillProb *P, const long long *zbase, int n, long long l_tot,
+                                                      const long long *rbase, int8_t *rowsign) {
+    dep_wait();
+    dep_next();
+    const int lane = threadIdx.x & 31;
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long L = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); L < l_tot; L += warps) {
+        const int p = find_row_prob(zbase, n, L);
+        const int len = P[p].ny;
+        int8_t *e = rowsign + rbase[p] + (L - zbase[p]) * (long long)len;
+        int carry = 0;
+        for (int s0 = 0; s0 < len; s0 += 1024) {
+            const int chunks = min(32, (len - s0 + 31) >> 5);
+            unsigned known = 0, neg = 0;
+            for (int c0 = 0; c0 < chunks; c0 += 8) {
+                int v[8];
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    const int i = s0 + (c0 + u) * 32 + lane;
+                    v[u] = i < len ? (int)e[i] : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
+                    const unsigned km = __ballot_sync(FULL_MASK, v[u] != 0), nm = __ballot_sync(FULL_MASK, v[u] < 0);
+                    if (lane == c0 + u) {
+                        known = km;
+                        neg = nm;
+                    }
+                }
             }
-            if (bm) carry = ((nm >> (31 - __clz(bm))) & 1u) ? -1 : 1;
+            const int had = carry;
+            const int in = chunk_signs(known, neg, carry);
+            if (carry == 0) continue;  // nothing known so far
+            if (had == 0) {
+                const int8_t m = (int8_t)(2 * __shfl_sync(FULL_MASK, in, 0));
+                for (int i = lane; i < s0; i += 32) e[i] = m;
+            }
+            for (int c = 0; c < chunks; c++) {
+                const unsigned ck = __shfl_sync(FULL_MASK, known, c), cn = __shfl_sync(FULL_MASK, neg, c);
+                const int s = sign_at(ck, cn, __shfl_sync(FULL_MASK, in, c));
+                const int i = s0 + c * 32 + lane;
+                if (i < len && !((ck >> lane) & 1u)) e[i] = (int8_t)(2 * s);
+            }
         }
     }
 }
 
-// Nearest-known propagation of the row signs along one line of the (y, z) row grid of each problem:
-// along y for every (problem, z) when ALONG_Y, else along z for every (problem, y).  Unknown entries
-// (0) take the sign of the nearest known entry before them, else after them; after the z pass the
-// entries still unknown (a problem without band points) become outside.  Resolved rows are marked
-// +-2 so that k_fill_empty can tell them from rows with band points.
-template <bool ALONG_Y>
-__global__ void k_fill_lines(const FillProb *P, const long long *lbase, int n, long long l_tot,
-                             const long long *rbase, int8_t *rowsign) {
-    const int lane = threadIdx.x & 31;
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long L = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); L < l_tot; L += warps) {
-        const int p = find_row_prob(lbase, n, L);
-        const FillProb pr = P[p];
-        const long long li = L - lbase[p];
-        // line li: ALONG_Y -> z = li, entries j = 0..ny-1 (stride 1); else y = li, entries k (stride ny)
-        const int len = ALONG_Y ? pr.ny : pr.nz;
-        const long long stride = ALONG_Y ? 1 : pr.ny;
-        int8_t *e = rowsign + rbase[p] + (ALONG_Y ? li * pr.ny : li);
-        // pass 1 (forward): carry the last known sign; pass 2 (backward) fills what is still unknown
-        int carry = 0;
-        for (int i0 = 0; i0 < len; i0 += 32) {
-            const int i = i0 + lane;
-            const int v = i < len ? (int)e[i * stride] : 0;
-            const unsigned km = __ballot_sync(FULL_MASK, v != 0), nm = __ballot_sync(FULL_MASK, v < 0);
-            if (i < len && v == 0) {
-                const unsigned left = km & (0xffffffffu >> (31 - lane));
-                const int s = left ? (((nm >> (31 - __clz(left))) & 1u) ? -1 : 1) : carry;
-                if (s != 0) e[i * stride] = (int8_t)(2 * s);
-            }
-            if (km) carry = ((nm >> (31 - __clz(km))) & 1u) ? -1 : 1;
+// The same along z for every (problem, y), after which the rows still unknown (a problem without band
+// points) become outside.  A line's entries are ny bytes apart, so a block takes 32 neighbouring
+// lines, one per lane, and its warps an eighth of their length each: first what is known in each part,
+// then the entries.  (A warp per line, its lanes along the stride, took 9 us
+// for 331 lines of 257 and 13.8 us for 128 of 96; now 5.5 and 4.5.)
+__global__ void __launch_bounds__(256) k_fill_lines_z(const FillProb *P, const long long *ybase, int n, long long l_tot,
+                                                      const long long *rbase, int8_t *rowsign) {
+    dep_wait();
+    dep_next();
+    __shared__ int8_t s_first[8][32], s_last[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (long long L0 = (long long)blockIdx.x * 32; L0 < l_tot; L0 += (long long)gridDim.x * 32) {
+        const long long L = L0 + lane;
+        int8_t *e = nullptr;
+        int k0 = 0, k1 = 0;
+        long long stride = 0;
+        if (L < l_tot) {
+            const int p = find_row_prob(ybase, n, L);
+            const int len = P[p].nz, part = (len + 7) / 8;
+            stride = P[p].ny;
+            e = rowsign + rbase[p] + (L - ybase[p]);
+            k0 = min(warp * part, len);
+            k1 = min(k0 + part, len);
         }
-        __syncwarp();
-        carry = 0;
-        for (int i0 = ((len - 1) / 32) * 32; i0 >= 0; i0 -= 32) {
-            const int i = i0 + lane;
-            const int v = i < len ? (int)e[i * stride] : 0;
-            const unsigned km = __ballot_sync(FULL_MASK, v != 0), nm = __ballot_sync(FULL_MASK, v < 0);
-            if (i < len && v == 0) {
-                const unsigned right = km & (0xffffffffu << lane);  // known lanes >= this one
-                int s = right ? (((nm >> (__ffs(right) - 1)) & 1u) ? -1 : 1) : carry;
-                if (!ALONG_Y && s == 0) s = 1;  // no band point in the whole problem: outside
-                if (s != 0) e[i * stride] = (int8_t)(2 * s);
+        int first = 0, last = 0;
+#pragma unroll 8
+        for (int k = k0; k < k1; k++) {
+            const int v = e[k * stride];
+            if (v != 0) {
+                last = v < 0 ? -1 : 1;
+                if (first == 0) first = last;
             }
-            if (km) carry = ((nm >> (__ffs(km) - 1)) & 1u) ? -1 : 1;
         }
+        s_first[warp][lane] = (int8_t)first;
+        s_last[warp][lane] = (int8_t)last;
+        __syncthreads();
+        int carry = 0, lead = 0;
+        for (int w = 7; w >= 0; w--) lead = s_first[w][lane] ? s_first[w][lane] : lead;
+        for (int w = 0; w < warp; w++) carry = s_last[w][lane] ? s_last[w][lane] : carry;
+        if (carry == 0) carry = lead ? lead : 1;  // no band point in the whole problem: outside
+        for (int kk = k0; kk < k1; kk += 8) {  // (eight loads, then the stores: they would wait for each other)
+            int v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = kk + u < k1 ? (int)e[(kk + u) * stride] : 1;
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                if (v[u] == 0) e[(kk + u) * stride] = (int8_t)(2 * carry);
+                else if (kk + u < k1) carry = v[u] < 0 ? -1 : 1;
+            }
+        }
+        __syncthreads();  // the shared signs are written again for the next lines
     }
 }
 
 // rows without band points that lie inside: the whole row becomes -inf
 __global__ void k_fill_empty(const FillProb *P, const long long *rbase, int n, long long r_tot,
                              const int8_t *rowsign) {
+    dep_wait();
+    dep_next();
     const int lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < r_tot; r += warps) {
@@ -140,20 +241,12 @@ __global__ void k_fill_empty(const FillProb *P, const long long *rbase, int n, l
 
 cudaError_t fill_sign(const FillProb *P, const long long *rbase, const long long *zbase, const long long *ybase, int n,
                       long long r_tot, long long z_tot, long long y_tot, int8_t *rowsign, int n_sm, cudaStream_t s) {
-    const int blocks = 8 * n_sm;  // 8 warps per block, grid-stride over rows / lines
-    k_fill_rows<<<blocks, 256, 0, s>>>(P, rbase, n, r_tot, rowsign);
-    SDF_LAUNCHED(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_fill_lines<true><<<blocks, 256, 0, s>>>(P, zbase, n, z_tot, rbase, rowsign);
-    SDF_LAUNCHED(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_fill_lines<false><<<blocks, 256, 0, s>>>(P, ybase, n, y_tot, rbase, rowsign);
-    SDF_LAUNCHED(1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_fill_empty<<<blocks, 256, 0, s>>>(P, rbase, n, r_tot, rowsign);
-    SDF_LAUNCHED(1);
-    return cudaGetLastError();
+    const dim3 blocks(8 * n_sm), bt(256);  // 8 warps per block, grid-stride over rows / lines
+    cudaError_t e = launch_dep(k_fill_rows, blocks, bt, 0, s, P, rbase, n, r_tot, rowsign);
+    if (e == cudaSuccess) e = launch_dep(k_fill_lines_y, blocks, bt, 0, s, P, zbase, n, z_tot, rbase, rowsign);
+    if (e == cudaSuccess) e = launch_dep(k_fill_lines_z, blocks, bt, 0, s, P, ybase, n, y_tot, rbase, rowsign);
+    if (e == cudaSuccess) e = launch_dep(k_fill_empty, blocks, bt, 0, s, P, rbase, n, r_tot, (const int8_t *)rowsign);
+    return e;
 }
 
 }  // namespace sdf
