@@ -427,12 +427,27 @@ __global__ void __launch_bounds__(BT) k_face_records(const int32_t *face_vid, co
                c = load_vpos(vpos, face_vid[3 * f + 2]);
         const double3 A = d3(a), E1 = d3(b) - A, E2 = d3(c) - A;
         const double3 CR = dcross3(E1, E2);
-        double len = sqrt(ddot3(CR, CR));
-        if (!(len > 1e-14 * (ddot3(E1, E1) + ddot3(E2, E2)))) {  // zero area (Section 4)
-            degenerate = true;
-            len = fmax(len, 1e-300);
+        const double q = ddot3(CR, CR);  // the square of twice the area
+        const float3 e1 = b - a, e2 = c - a;
+        const float lsq = dot3(e1, e1) + dot3(e2, e2), qf = (float)q;
+        double inv;
+        if (lsq > 1e-12f && qf > 1e-16f * lsq * lsq && qf > 1e-30f && qf < 1e30f) {
+            // clearly not degenerate, and within FP32's range: 1 / sqrt(q) by Newton's iteration from the
+            // FP32 value (relative error 1e-7, then 2e-14, then rounding); the exact square root and
+            // quotient are long sequences on the FP64 pipe, which bounds this kernel (241 us for 2.1 M
+            // triangles with them, 193 without)
+            inv = (double)rsqrtf(qf);
+#pragma unroll
+            for (int it = 0; it < 2; it++) inv = fma(inv * 0.5, fma(-q * inv, inv, 1.0), inv);
+        } else {
+            double len = sqrt(q);
+            if (!(len > 1e-14 * (ddot3(E1, E1) + ddot3(E2, E2)))) {  // zero area (Section 4)
+                degenerate = true;
+                len = fmax(len, 1e-300);
+            }
+            inv = 1.0 / len;
         }
-        const double3 N = (1.0 / len) * CR;
+        const double3 N = inv * CR;
         const float3 n = make_float3((float)N.x, (float)N.y, (float)N.z);
         // plane of the face, and the three side planes with inward normals n x (edge) (Section 8.1)
         face_rec[4 * f + 0] = make_float4(n.x, n.y, n.z, (float)-ddot3(N, A));
