@@ -1046,6 +1046,23 @@ constexpr int SPLIT_MIN = 2048, SPLIT_MAX = 8192, SPLIT_PAIRS = 1024, SPLIT_MAX_
 static_assert(offsetof(DevCounters, n_split_items) == offsetof(DevCounters, tile_hist) + 33 * sizeof(unsigned),
               "the per-launch tile-list counters must be contiguous");
 
+// a band tile's entry in the band list: the tile, or -1 and its items in split_items
+__device__ __forceinline__ int32_t band_entry(int64_t t, uint32_t np, uint32_t total, DevCounters *ctr,
+                                              int2 *split_items, int split_cap, int n_ctas) {
+    int32_t entry = (int32_t)t;
+    const uint32_t split_from = min(max(total / (uint32_t)n_ctas, (uint32_t)SPLIT_MIN), (uint32_t)SPLIT_MAX);
+    if (np > split_from && split_cap > 0) {
+        const unsigned slot = atomicAdd(&ctr->n_split, 1u);
+        if (slot < (unsigned)split_cap) {
+            const int S = (int)min((np + SPLIT_PAIRS - 1) / SPLIT_PAIRS, (uint32_t)SPLIT_MAX_ITEMS);
+            const unsigned base = atomicAdd(&ctr->n_split_items, (unsigned)S);  // < split_cap * SPLIT_MAX_ITEMS
+            for (int i = 0; i < S; i++) split_items[base + i] = make_int2((int)t, (int)(slot | i << 12 | S << 20));
+            entry = -1;
+        }
+    }
+    return entry;
+}
+
 __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const uint32_t *band_pos,
                              int32_t *band_list, int32_t *empty_list, DevCounters *ctr, int lpt, int2 *split_items,
                              int split_cap, int n_ctas) {
@@ -1058,17 +1075,7 @@ __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const u
         empty_list[t - band_pos[t]] = (int32_t)t;
         return;
     }
-    int32_t entry = (int32_t)t;
-    const uint32_t split_from = min(max(bin_start[3 * n_tiles] / (uint32_t)n_ctas, (uint32_t)SPLIT_MIN), (uint32_t)SPLIT_MAX);
-    if (np > split_from && split_cap > 0) {
-        const unsigned slot = atomicAdd(&ctr->n_split, 1u);
-        if (slot < (unsigned)split_cap) {
-            const int S = (int)min((np + SPLIT_PAIRS - 1) / SPLIT_PAIRS, (uint32_t)SPLIT_MAX_ITEMS);
-            const unsigned base = atomicAdd(&ctr->n_split_items, (unsigned)S);  // < split_cap * SPLIT_MAX_ITEMS
-            for (int i = 0; i < S; i++) split_items[base + i] = make_int2((int)t, (int)(slot | i << 12 | S << 20));
-            entry = -1;
-        }
-    }
+    const int32_t entry = band_entry(t, np, bin_start[3 * n_tiles], ctr, split_items, split_cap, n_ctas);
     if (!lpt) {
         band_list[band_pos[t]] = entry;
     } else {
@@ -1076,6 +1083,68 @@ __global__ void k_tile_lists(const uint32_t *bin_start, int64_t n_tiles, const u
         uint32_t base = 0;
         for (int k = 0; k < c; k++) base += ctr->tile_hist[k];
         band_list[base + atomicAdd(&ctr->tile_cursor[c], 1u)] = entry;
+    }
+}
+
+// The work list of a launch over at most LISTS_ONE tiles in one block, instead of k_band_flags, a scan
+// and k_tile_lists: on a few hundred tiles each of the three takes 2 us, nearly all of it launch and
+// memory latency, and this one 2.9; at 8192 tiles they take 8 us either way (two launches fewer).  A
+// thread has up to 8 consecutive tiles.
+constexpr int64_t LISTS_ONE = 8192;
+constexpr int LISTS_NT = 1024;
+__global__ void __launch_bounds__(LISTS_NT) k_tile_lists_one(const uint32_t *bin_start, int n_tiles, uint32_t *n_band,
+                                                             int32_t *band_list, int32_t *empty_list, DevCounters *ctr,
+                                                             int lpt, int2 *split_items, int split_cap, int n_ctas) {
+    dep_wait();
+    dep_next();
+    __shared__ uint32_t s_warp[32], s_class[N_COST_CLASSES];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int per = (n_tiles + LISTS_NT - 1) / LISTS_NT, t0 = t * per;
+    if (t < N_COST_CLASSES) s_class[t] = 0;
+    uint32_t st[LISTS_ONE / LISTS_NT + 1];
+#pragma unroll
+    for (int k = 0; k <= (int)(LISTS_ONE / LISTS_NT); k++) st[k] = bin_start[3 * min(t0 + min(k, per), n_tiles)];
+    uint32_t mine = 0;
+#pragma unroll
+    for (int k = 0; k < (int)(LISTS_ONE / LISTS_NT); k++) mine += st[k + 1] != st[k];
+    const uint32_t incl = (uint32_t)warp_incl_scan((int)mine);
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t v = s_warp[lane], vi = (uint32_t)warp_incl_scan((int)v);
+        s_warp[lane] = vi - v;
+        if (lane == 31) *n_band = vi;
+    }
+    if (lpt) {
+#pragma unroll
+        for (int k = 0; k < (int)(LISTS_ONE / LISTS_NT); k++)
+            if (st[k + 1] != st[k]) atomicAdd(&s_class[tile_cost_class(st[k + 1] - st[k])], 1u);
+    }
+    __syncthreads();
+    uint32_t pos = s_warp[warp] + incl - mine;  // band tiles before this thread's
+    if (lpt && t < N_COST_CLASSES) {  // (one warp) each class's first place
+        uint32_t c = s_class[t], inc = c;
+#pragma unroll
+        for (int o = 1; o < N_COST_CLASSES; o <<= 1) {
+            const uint32_t v = __shfl_up_sync((1u << N_COST_CLASSES) - 1u, inc, o);
+            if (t >= o) inc += v;
+        }
+        s_class[t] = inc - c;
+    }
+    __syncthreads();
+    const uint32_t total = bin_start[3 * n_tiles];
+#pragma unroll
+    for (int k = 0; k < (int)(LISTS_ONE / LISTS_NT); k++) {
+        const int tile = t0 + k;
+        const uint32_t np = st[k + 1] - st[k];
+        if (k >= per || tile >= n_tiles) continue;
+        if (!np) {
+            empty_list[tile - (int)pos] = tile;
+            continue;
+        }
+        const int32_t entry = band_entry(tile, np, total, ctr, split_items, split_cap, n_ctas);
+        band_list[lpt ? atomicAdd(&s_class[tile_cost_class(np)], 1u) : pos] = entry;
+        pos++;
     }
 }
 
@@ -2670,15 +2739,22 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
     SDF_TRY(scan_exclusive_u32(sc.cnt, sc.start, n_bins, true, sc.scan_tmp, s, &sc.ctr->nb_status));
     SDF_TRY(launch_dep(sc.boxes ? k_bin<BIN_FILL, TY, TZ> : k_bin<BIN_FILL_AGAIN, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
                        f_tot, sc.cnt, (const uint32_t *)sc.start, sc.pairs, sc.pair_cap, sc.ctr, sc.boxes));
-    // band / empty tile lists for the persistent tile kernel (one scan of the band flags)
-    uint32_t *flags = sc.cnt;  // the fill cursors are no longer needed
+    // band / empty tile lists for the persistent tile kernel
     const int lpt = n > 1;  // largest-first order of the band tiles for batches
-    SDF_TRY(launch_dep(k_band_flags, dim3(nblk(n_tiles, 256)), dim3(256), 0, s, (const uint32_t *)sc.start, n_tiles,
-                       flags, sc.ctr, lpt));
-    SDF_TRY(scan_exclusive_u32(flags, sc.band_pos, n_tiles, true, sc.scan_tmp, s, &sc.ctr->nb_status));
-    SDF_TRY(launch_dep(k_tile_lists, dim3(nblk(n_tiles, 256)), dim3(256), 0, s, (const uint32_t *)sc.start, n_tiles,
-                       (const uint32_t *)sc.band_pos, sc.band_list, sc.empty_list, sc.ctr, lpt, sc.split_items,
-                       sc.split_items ? SPLIT_SLOTS : 0, 4 * num_sms()));
+    const int split_cap = sc.split_items ? SPLIT_SLOTS : 0;
+    if (n_tiles <= LISTS_ONE) {
+        SDF_TRY(launch_dep(k_tile_lists_one, dim3(1), dim3(LISTS_NT), 0, s, (const uint32_t *)sc.start, (int)n_tiles,
+                           sc.band_pos + n_tiles, sc.band_list, sc.empty_list, sc.ctr, lpt, sc.split_items, split_cap,
+                           4 * num_sms()));
+    } else {  // one scan of the band flags
+        uint32_t *flags = sc.cnt;  // the fill cursors are no longer needed
+        SDF_TRY(launch_dep(k_band_flags, dim3(nblk(n_tiles, 256)), dim3(256), 0, s, (const uint32_t *)sc.start, n_tiles,
+                           flags, sc.ctr, lpt));
+        SDF_TRY(scan_exclusive_u32(flags, sc.band_pos, n_tiles, true, sc.scan_tmp, s, &sc.ctr->nb_status));
+        SDF_TRY(launch_dep(k_tile_lists, dim3(nblk(n_tiles, 256)), dim3(256), 0, s, (const uint32_t *)sc.start, n_tiles,
+                           (const uint32_t *)sc.band_pos, sc.band_list, sc.empty_list, sc.ctr, lpt, sc.split_items,
+                           split_cap, 4 * num_sms()));
+    }
     Outputs o;
     o.pairs = sc.pairs;
     o.bin_start = sc.start;

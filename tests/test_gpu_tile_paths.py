@@ -56,3 +56,24 @@ def test_small_launches_equal_a_large_batch():
         a, b = _sorted(bl.entries[:n]), _sorted(bl1.entries[:n])
         assert torch.equal(a, b)
         assert torch.equal(win1.reshape(-1).cpu().long()[a[:, 0]], a[:, 1])
+
+
+@pytest.mark.parametrize("make", [lambda: meshgen.torus(nu=120, nv=48, seed=5),
+                                  lambda: meshgen.dense_cluster(freq_big=3, freq_small=30)])
+def test_work_list_in_one_block(make):
+    """Launches over at most 8192 tiles list them in one block: 8192 tiles against the same layers of
+    8448 (three launches), one problem and a batch (listed by cost class), down to a single tile."""
+    feats = sdf.sdf_build_features(torch.from_numpy(make().soup(seed=2)).cuda())
+    h = 1.0 / 512
+    origin = (0.0, 0.5 - 64 * h, 0.5 - 128 * h)
+    one = sdf.Grid(512, 128, 256, origin, h)
+    more = sdf.Grid(512, 128, 264, origin, h)
+    w = 3 * h
+    d1, w1 = sdf.sdf_narrow_band(feats, one, w, winner=True)
+    d2, w2 = sdf.sdf_narrow_band(feats, more, w, winner=True)
+    assert torch.isfinite(d1).any()
+    assert torch.equal(d1, d2[:256]) and torch.equal(w1, w2[:256])
+    grids = [sdf.Grid(512, 128, 128, origin, h), sdf.Grid(512, 128, 100, origin, h, k0=128), sdf.Grid(20, 5, 3, origin, h)]
+    d3 = sdf.sdf_narrow_band([feats] * 3, grids, [w] * 3)
+    assert torch.equal(d3[0], d1[:128]) and torch.equal(d3[1], d1[128:228]) and torch.equal(d3[2], d1[:3, :5, :20])
+    assert torch.equal(sdf.sdf_narrow_band(feats, grids[2], w), d1[:3, :5, :20])
