@@ -8,9 +8,10 @@
 // vertices serially inside each equal-code run.  Here the sort key is 40 bits (five 8-bit radix
 // passes): the 30-bit Morton code of the quantised position (over the soup's bounding box,
 // Section 7.1) in the high bits and a 10-bit hash of the exact coordinate bits in the low bits, so
-// equal vertices always share a key and distinct vertices rarely do.  Runs of equal keys holding different coordinates (hash
-// collisions, or distinct vertices in one Morton cell) are re-ordered by exact coordinates by one
-// thread per such run, the only serial step left of the paper's fix-up.
+// equal vertices always share a key and distinct vertices rarely do.  Runs of equal keys holding
+// different coordinates (hash collisions, or distinct vertices in one Morton cell) are listed and
+// re-ordered by exact coordinates, short ones by one thread each, the only serial step left of the
+// paper's fix-up.
 //
 // Edge pairing (Section 7.1): the twin of the directed edge a->b is the corner of b whose next
 // vertex is a, found in b's fan of the vertex CSR; a->b must occur once around a and b->a once
@@ -133,37 +134,63 @@ __device__ __forceinline__ bool less_xyz(const float *soup, uint32_t a, uint32_t
     return a < b;
 }
 
-// One thread per run of equal keys.  A run that mixes distinct coordinates (a hash collision, or
-// distinct vertices in one Morton cell, as in a dense cluster of small triangles) is re-ordered by
-// (coordinate bits, soup index) so that equal vertices become contiguous: runs of up to
-// WELD_SHORT entries by the thread itself (insertion sort), longer ones are listed for
-// k_weld_sort_runs, one block per run.
-constexpr int WELD_SHORT = 32, WELD_BLOCK_MAX = 2048;
-__global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *soup, int64_t n, int2 *long_runs,
-                           int64_t long_cap, unsigned *n_long) {
+// head[i] = 1 where a sorted entry differs from the one before it.  A run of equal keys that mixes
+// distinct coordinates (a hash collision, or distinct vertices in one Morton cell, as in a dense cluster
+// of small triangles) has to be put in order first: it is listed, once, by the first of its entries that
+// differs from its predecessor.  Bound by the gather of the coordinates, one entry per thread; a
+// thread per run walking its entries before this pass took another 115 us on 6.3 M entries.
+__global__ void k_weld_heads(const uint64_t *keys, const uint32_t *vals, const float *soup, int64_t n,
+                             uint32_t *head, int32_t *mixed, unsigned *n_mixed) {
     dep_wait();
     dep_next();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n || (i > 0 && keys[i] == keys[i - 1])) return;
-    int64_t e = i + 1;
-    bool mixed = false;
-    while (e < n && keys[e] == keys[i]) {
-        mixed |= !same_xyz(soup, vals[e], vals[i]);
-        e++;
+    if (i >= n) return;
+    const bool eq = i > 0 && keys[i] == keys[i - 1];
+    const bool same = eq && same_xyz(soup, vals[i], vals[i - 1]);
+    head[i] = same ? 0u : 1u;
+    if (!eq || same) return;
+    int64_t q = i - 1;  // back to the run's start, while all before are equal
+    while (q > 0 && keys[q - 1] == keys[q]) {
+        if (!same_xyz(soup, vals[q], vals[q - 1])) return;  // not the first
+        q--;
     }
-    if (!mixed) return;
-    if (e - i > WELD_SHORT && e - i <= WELD_BLOCK_MAX) {
-        const unsigned slot = atomicAdd(n_long, 1u);
-        if ((int64_t)slot < long_cap) {
-            long_runs[slot] = make_int2((int)i, (int)(e - i));
-            return;
+    mixed[atomicAdd(n_mixed, 1u)] = (int32_t)q;  // a mixed run has at least two entries: at most n / 2 of them
+}
+
+// the heads of a run put in order
+__device__ __forceinline__ void run_heads(const uint32_t *vals, const float *soup, int64_t i, int64_t e, int64_t from,
+                                          int64_t step, uint32_t *head) {
+    for (int64_t a = i + 1 + from; a < e; a += step) head[a] = same_xyz(soup, vals[a], vals[a - 1]) ? 0u : 1u;
+}
+
+// The mixed runs (grid-stride over the device-side count): re-ordered by (coordinate bits, soup index)
+// so that equal vertices become contiguous, runs of up to WELD_SHORT entries by the thread itself
+// (insertion sort), longer ones are listed for k_weld_sort_runs, one block per run.
+constexpr int WELD_SHORT = 32, WELD_BLOCK_MAX = 2048;
+__global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *soup, int64_t n, const int32_t *mixed,
+                           const unsigned *n_mixed, uint32_t *head, int2 *long_runs, int64_t long_cap,
+                           unsigned *n_long) {
+    dep_wait();
+    dep_next();
+    const int64_t nm = *n_mixed;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nm; r += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = mixed[r];
+        int64_t e = i + 1;
+        while (e < n && keys[e] == keys[i]) e++;
+        if (e - i > WELD_SHORT && e - i <= WELD_BLOCK_MAX) {
+            const unsigned slot = atomicAdd(n_long, 1u);
+            if ((int64_t)slot < long_cap) {
+                long_runs[slot] = make_int2((int)i, (int)(e - i));
+                continue;
+            }
         }
-    }
-    for (int64_t a = i + 1; a < e; a++) {  // short runs (and runs beyond the block sort's size)
-        uint32_t v = vals[a];
-        int64_t b = a - 1;
-        while (b >= i && less_xyz(soup, v, vals[b])) { vals[b + 1] = vals[b]; b--; }
-        vals[b + 1] = v;
+        for (int64_t a = i + 1; a < e; a++) {  // short runs (and runs beyond the block sort's size)
+            uint32_t v = vals[a];
+            int64_t b = a - 1;
+            while (b >= i && less_xyz(soup, v, vals[b])) { vals[b + 1] = vals[b]; b--; }
+            vals[b + 1] = v;
+        }
+        run_heads(vals, soup, i, e, 0, 1, head);
     }
 }
 
@@ -172,7 +199,7 @@ __global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *so
 // the next power of two (padding sorts last), then written back.  Any total order of the
 // coordinate bits makes equal vertices contiguous; -0 is read as +0.
 __global__ void __launch_bounds__(256) k_weld_sort_runs(const int2 *long_runs, const unsigned *n_long, int64_t long_cap,
-                                                        uint32_t *vals, const float *soup) {
+                                                        uint32_t *vals, const float *soup, uint32_t *head) {
     dep_wait();
     dep_next();
     __shared__ uint4 rec[WELD_BLOCK_MAX];
@@ -210,16 +237,8 @@ __global__ void __launch_bounds__(256) k_weld_sort_runs(const int2 *long_runs, c
         }
         for (int t = threadIdx.x; t < run.y; t += blockDim.x) vals[run.x + t] = rec[t].w;
         __syncthreads();
+        run_heads(vals, soup, run.x, run.x + (int64_t)run.y, threadIdx.x, blockDim.x, head);
     }
-}
-
-__global__ void k_weld_heads(const uint64_t *keys, const uint32_t *vals, const float *soup, int64_t n,
-                             uint32_t *head) {
-    dep_wait();
-    dep_next();
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    head[i] = (i == 0 || keys[i] != keys[i - 1] || !same_xyz(soup, vals[i], vals[i - 1])) ? 1u : 0u;
 }
 
 // head[] holds the exclusive scan of the run heads; vid = that + is_head - 1
@@ -820,7 +839,7 @@ __global__ void k_build_init(unsigned *ctr, int64_t ctr_words, float *bb, unsign
     for (int64_t i = threadIdx.x; i < ctr_words; i += blockDim.x) ctr[i] = 0u;
     for (int64_t i = threadIdx.x; i < scan_words; i += blockDim.x) scan[i] = 0u;
     if (threadIdx.x < 6) bb[threadIdx.x] = threadIdx.x < 3 ? INFINITY : -INFINITY;
-    if (threadIdx.x == 0) *n_long = 0u;
+    if (threadIdx.x < 2) n_long[threadIdx.x] = 0u;  // and the mixed runs' count
 }
 
 // grid of a records kernel over n threads' worth of items: the blocks resident on the device at
@@ -994,7 +1013,8 @@ extern "C" int sdf_build_features(const float *soup, int64_t n_tri, uint32_t fla
     size_t off_keys = 0, off_kalt = off_keys + 8 * n, off_vals = off_kalt + 8 * n, off_valt = off_vals + 4 * n,
            off_head = off_valt + 4 * n, off_bb = off_head + 4 * (n + 1) + 64,
            off_long = (off_bb + 64 + 15) & ~(size_t)15,               // int2: 8-byte aligned (16 here)
-           off_rtmp = (off_long + 8 * long_cap + 64 + 15) & ~(size_t)15;
+           off_mixed = (off_long + 8 * long_cap + 64 + 15) & ~(size_t)15,  // at most n / 2 mixed runs
+           off_rtmp = (off_mixed + 4 * (n / 2 + 1) + 64 + 15) & ~(size_t)15;
     // one scan state for the build's scans and sorts, cleared once here (see scan_exclusive_u32)
     const size_t scan_bytes = std::max(scan_state_bytes(n + 1), radix_scan_state_bytes(n));
     const size_t off_scan = (off_rtmp + radix_tmp_bytes(n) + 255) & ~(size_t)255;
@@ -1006,7 +1026,9 @@ extern "C" int sdf_build_features(const float *soup, int64_t n_tri, uint32_t fla
     uint32_t *head = reinterpret_cast<uint32_t *>(base + off_head);
     float *bb = reinterpret_cast<float *>(base + off_bb);
     unsigned *n_long = reinterpret_cast<unsigned *>(base + off_bb + 32);
+    unsigned *n_mixed = n_long + 1;
     int2 *long_runs = reinterpret_cast<int2 *>(base + off_long);
+    int32_t *mixed = reinterpret_cast<int32_t *>(base + off_mixed);
     void *rtmp = base + off_rtmp;
     void *scan_state = base + off_scan;
 
@@ -1021,9 +1043,10 @@ extern "C" int sdf_build_features(const float *soup, int64_t n_tri, uint32_t fla
                      0, s, soup, n, bb, f->ctr));
     B_TRY(launch_dep(k_weld_keys, dim3(nblk(n)), dim3(BT), 0, s, soup, n, bb, keys, vals));
     B_TRY(radix_sort_u64(keys, vals, kalt, valt, n, 40, rtmp, scan_state, s, err));
-    B_TRY(launch_dep(k_weld_fix, dim3(nblk(n)), dim3(BT), 0, s, keys, vals, soup, n, long_runs, long_cap, n_long));
-    B_TRY(launch_dep(k_weld_sort_runs, dim3(2 * 152), dim3(256), 0, s, long_runs, n_long, long_cap, vals, soup));
-    B_TRY(launch_dep(k_weld_heads, dim3(nblk(n)), dim3(BT), 0, s, keys, vals, soup, n, valt));
+    B_TRY(launch_dep(k_weld_heads, dim3(nblk(n)), dim3(BT), 0, s, keys, vals, soup, n, valt, mixed, n_mixed));
+    B_TRY(launch_dep(k_weld_fix, dim3((unsigned)std::min<int64_t>(nblk(n / 2 + 1), 2 * 152)), dim3(BT), 0, s, keys, vals,
+                     soup, n, mixed, n_mixed, valt, long_runs, long_cap, n_long));
+    B_TRY(launch_dep(k_weld_sort_runs, dim3(2 * 152), dim3(256), 0, s, long_runs, n_long, long_cap, vals, soup, valt));
     // head[i] = number of run heads before i, head[n] = V (so head[i+1] is the inclusive count at i)
     B_TRY(scan_exclusive_u32(valt, head, n, true, scan_state, s, err));
     uint32_t Vh = 0;

@@ -461,7 +461,7 @@ int rs_items(int64_t n) {
 }
 
 template <int ITEMS>
-cudaError_t rs_passes(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, int64_t n, int bits,
+cudaError_t rs_passes(uint64_t *&keys, uint32_t *&vals, uint64_t *&keys_alt, uint32_t *&vals_alt, int64_t n, int bits,
                       void *tmp, void *scan_state, cudaStream_t s, unsigned *err) {
     static bool attr_set = false;
     if (!attr_set) {
@@ -489,11 +489,11 @@ cudaError_t rs_passes(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32
         uint64_t *tk = ki; ki = ko; ko = tk;
         uint32_t *tv = vi; vi = vo; vo = tv;
     }
-    if (ki != keys) {
-        cudaError_t e = cudaMemcpyAsync(keys, ki, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(vals, vi, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
+    if (ki != keys) {  // an odd number of passes ends in the alternates: they change roles
+        keys_alt = keys;
+        vals_alt = vals;
+        keys = ki;
+        vals = vi;
     }
     return cudaSuccess;
 }
@@ -563,7 +563,7 @@ size_t radix_scan_state_bytes(int64_t n) {
     return scan_state_bytes(((n + tile - 1) / tile) * RADIX);
 }
 
-cudaError_t radix_sort_u64(uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, int64_t n,
+cudaError_t radix_sort_u64(uint64_t *&keys, uint32_t *&vals, uint64_t *&keys_alt, uint32_t *&vals_alt, int64_t n,
                            int bits, void *tmp, void *scan_state, cudaStream_t s, unsigned *err) {
     if (n <= 1 || bits <= 0) return cudaSuccess;
     const int items = rs_items(n);
