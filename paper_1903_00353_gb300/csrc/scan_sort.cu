@@ -311,7 +311,14 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t *kin, 
 // needs no second buffer; grid barrier (the next pass reads what the others wrote).  Data written
 // by other CTAs is read past L1 (ld.global.cg).  Against the three launches per pass above (a
 // histogram, a scan and a scatter) this makes 1 launch per sort.
+//
+// With at most RS_DIRECT tiles step (2) and its barrier are left out: each CTA reads all tiles' counts
+// itself (1 KB per tile, tile-major, sixteen loads in flight) and sums them per digit.  A pass is then
+// bound by two barriers, about 1.5 us each, and the latency of its loads; five passes over 64 tiles (the
+// weld of 10,800 triangles) took 60 us with three barriers, now 42.  For more tiles the counts that
+// every CTA reads grow with the square of their number (147 tiles: 119 us against 63).
 constexpr unsigned RS_POLL_LIMIT = 1u << 20;
+constexpr unsigned RS_DIRECT = 128;
 
 // Grid barrier of a cooperative launch on bar[0] (arrivals, 0 between barriers) and bar[1]
 // (generation): the last CTA to arrive clears the arrivals and advances the generation; the others
@@ -373,6 +380,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_one(uint64_t *keys, uint32_t 
     const int cnt = (int)(n - tile0 < (int64_t)TILE ? n - tile0 : (int64_t)TILE);
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint32_t *mycnt = wcnt + warp * RADIX;
+    const bool direct = nb <= RS_DIRECT && n < 65536;
     for (int p = 0; p < passes; p++) {
         const int shift = 8 * p;
         // (1) ranks within the tile: lanes in order within a warp, warps in order (stable)
@@ -402,29 +410,49 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_one(uint64_t *keys, uint32_t 
                 wcnt[w * RADIX + threadIdx.x] = run;
                 run += c;
             }
-            counts[(int64_t)threadIdx.x * nb + t] = run;
+            counts[direct ? (int64_t)t * RADIX + threadIdx.x : (int64_t)threadIdx.x * nb + t] = run;
             bstart[threadIdx.x] = block_excl_scan_u32(run, &s_tot);
         }
         if (!grid_barrier(bar, ++target, err)) return;
-        // (2) exclusive scan of digit d's counts over the tiles, in place, and the digit's total
-        for (unsigned d = t; d < (unsigned)RADIX; d += nb) {
-            uint32_t *row = counts + (int64_t)d * nb;
-            const unsigned per = (nb + RS_THREADS - 1) / RS_THREADS;
-            const unsigned j0 = min(threadIdx.x * per, nb), j1 = min(j0 + per, nb);
-            uint32_t s = 0;
-            for (unsigned j = j0; j < j1; j++) s += __ldcg(row + j);
-            uint32_t run = block_excl_scan_u32(s, &s_tot);
-            for (unsigned j = j0; j < j1; j++) {
-                const uint32_t c = __ldcg(row + j);
-                row[j] = run;
-                run += c;
+        if (!direct) {
+            // (2) exclusive scan of digit d's counts over the tiles, in place, and the digit's total
+            for (unsigned d = t; d < (unsigned)RADIX; d += nb) {
+                uint32_t *row = counts + (int64_t)d * nb;
+                const unsigned per = (nb + RS_THREADS - 1) / RS_THREADS;
+                const unsigned j0 = min(threadIdx.x * per, nb), j1 = min(j0 + per, nb);
+                uint32_t s = 0;
+                for (unsigned j = j0; j < j1; j++) s += __ldcg(row + j);
+                uint32_t run = block_excl_scan_u32(s, &s_tot);
+                for (unsigned j = j0; j < j1; j++) {
+                    const uint32_t c = __ldcg(row + j);
+                    row[j] = run;
+                    run += c;
+                }
+                if (threadIdx.x == 0) totals[d] = s_tot;
             }
-            if (threadIdx.x == 0) totals[d] = s_tot;
+            if (!grid_barrier(bar, ++target, err)) return;
         }
-        if (!grid_barrier(bar, ++target, err)) return;
         // (3) global start of the tile's run of digit d: the totals of the smaller digits plus the
         // counts of digit d in the tiles before this one
-        {
+        if (direct) {  // four digits per thread, a quarter of the tiles; (all << 16 | before) fits: n < 2^16
+            uint32_t *part = reinterpret_cast<uint32_t *>(skey);  // [4][RADIX], free until the scatter
+            const unsigned dq = threadIdx.x & 63, quarter = threadIdx.x >> 6;
+            uint4 sum = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 16
+            for (unsigned j = quarter; j < nb; j += 4) {
+                const uint4 c = __ldcg(reinterpret_cast<const uint4 *>(counts + (int64_t)j * RADIX) + dq);
+                const uint32_t m = j < t ? 0x10001u : 0x10000u;
+                sum.x += c.x * m;
+                sum.y += c.y * m;
+                sum.z += c.z * m;
+                sum.w += c.w * m;
+            }
+            *reinterpret_cast<uint4 *>(part + quarter * RADIX + 4 * dq) = sum;
+            __syncthreads();
+            const uint32_t v = part[threadIdx.x] + part[RADIX + threadIdx.x] + part[2 * RADIX + threadIdx.x] +
+                               part[3 * RADIX + threadIdx.x];
+            gofs[threadIdx.x] = block_excl_scan_u32(v >> 16, &s_tot) + (v & 0xffffu);
+        } else {
             const uint32_t start = block_excl_scan_u32(__ldcg(totals + threadIdx.x), &s_tot);
             gofs[threadIdx.x] = start + __ldcg(counts + (int64_t)threadIdx.x * nb + t);
         }
