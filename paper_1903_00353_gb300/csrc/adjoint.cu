@@ -317,6 +317,8 @@ __device__ __forceinline__ void adjoint_batch(const AdjArgs &a, const long long 
 
 template <bool F64>
 __global__ void __launch_bounds__(256) k_adjoint(AdjArgs a, int vec) {
+    dep_wait();
+    dep_next();
     __shared__ long long s_idx[8][ADJ_RING];
     __shared__ int s_wid[8][ADJ_RING];
     const int warp = threadIdx.x >> 5;
@@ -371,6 +373,8 @@ template <bool F64>
 __global__ void __launch_bounds__(256) k_adjoint_list(AdjArgs a, const uint2 *list, const unsigned long long *count,
                                                       long long cap, const float *dist, const float *target,
                                                       double *loss, unsigned long long *band_out) {
+    dep_wait();
+    dep_next();
     const long long n = min((long long)*count, cap);
     const int lane = threadIdx.x & 31;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -473,14 +477,9 @@ int list_adjoint(sdf_features_s *f, const sdf_grid *grid, const sdf_band_entry *
         SDF_TRY(cudaEventRecord(f->ev[4], s));
     }
     // the length is known on the device only: a grid of 8 CTAs per SM strides over the list
-    if (f64)
-        k_adjoint_list<true><<<8 * n_sm, 256, 0, s>>>(a, reinterpret_cast<const uint2 *>(list), list_count,
-                                                       (long long)list_cap, dist, target, loss_out, band_out);
-    else
-        k_adjoint_list<false><<<8 * n_sm, 256, 0, s>>>(a, reinterpret_cast<const uint2 *>(list), list_count,
-                                                        (long long)list_cap, dist, target, loss_out, band_out);
-    SDF_LAUNCHED(1);
-    SDF_TRY(cudaGetLastError());
+    SDF_TRY(launch_dep(f64 ? k_adjoint_list<true> : k_adjoint_list<false>, dim3(8 * n_sm), dim3(256), 0, s, a,
+                       reinterpret_cast<const uint2 *>(list), list_count, (long long)list_cap, dist, target, loss_out,
+                       band_out));
     if (!f64)
         SDF_TRY(launch_dep(k_grad_out, dim3((unsigned)((f->V + 255) / 256)), dim3(256), 0, s, f->grad4,
                            grad_vertices, (int64_t)f->V));
@@ -554,12 +553,7 @@ extern "C" int sdf_narrow_band_backward(const sdf_features *feats, const sdf_gri
             SDF_TRY_ST(resolve_timing(f));
             SDF_TRY(cudaEventRecord(f->ev[4], s));
         }
-        if (f64)
-            k_adjoint<true><<<(unsigned)blocks, 256, 0, s>>>(a, vec);
-        else
-            k_adjoint<false><<<(unsigned)blocks, 256, 0, s>>>(a, vec);
-        SDF_LAUNCHED(1);
-        SDF_TRY(cudaGetLastError());
+        SDF_TRY(launch_dep(f64 ? k_adjoint<true> : k_adjoint<false>, dim3((unsigned)blocks), dim3(256), 0, s, a, vec));
         if (!f64)
             SDF_TRY(launch_dep(k_grad_out, dim3((unsigned)((f->V + 255) / 256)), dim3(256), 0, s, f->grad4,
                                grad_vertices[p], (int64_t)f->V));
@@ -579,6 +573,8 @@ namespace sdf {
 namespace {
 __global__ void __launch_bounds__(256) k_band_l2(const float *dist, const float *target, int64_t n, float *grad,
                                                  double *loss, unsigned long long *band, int vec) {
+    dep_wait();
+    dep_next();
     double acc = 0.0;
     unsigned cnt = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -658,8 +654,7 @@ extern "C" int sdf_band_l2_loss(const float *dist, const float *target, int64_t 
     int64_t blocks = (n / (vec ? 4 : 1) + 255) / 256;
     if (blocks > 8 * (int64_t)n_sm) blocks = 8 * (int64_t)n_sm;
     if (blocks < 1) blocks = 1;
-    k_band_l2<<<(unsigned)blocks, 256, 0, s>>>(dist, target, n, grad_out, loss_out, band_out, vec);
-    SDF_LAUNCHED(1);
-    SDF_TRY(cudaGetLastError());
+    SDF_TRY(launch_dep(k_band_l2, dim3((unsigned)blocks), dim3(256), 0, s, dist, target, n, grad_out, loss_out, band_out,
+                       vec));
     return SDF_OK;
 }

@@ -842,6 +842,19 @@ __global__ void k_build_init(unsigned *ctr, int64_t ctr_words, float *bb, unsign
     if (threadIdx.x < 2) n_long[threadIdx.x] = 0u;  // and the mixed runs' count
 }
 
+// What the records kernels count up is cleared before new positions: class counts, status, precision
+// terms and box moments, in one dependent launch (four memsets before, each of which ended the chain of
+// dependent launches and cost 1 to 2 us).
+__global__ void k_positions_init(DevCounters *ctr) {
+    dep_wait();
+    dep_next();
+    const int t = threadIdx.x;
+    if (t < 8) ctr->cls[t] = 0;
+    if (t < 4) ctr->prec[t] = 0;
+    if (t < 7) ctr->box_mom[t] = 0.0;
+    if (t == 0) ctr->status = 0;
+}
+
 // grid of a records kernel over n threads' worth of items: the blocks resident on the device at
 // once (a single wave of the grid-stride loop), fewer when the items need fewer
 template <class K> unsigned rec_grid(K kernel, int64_t n) {
@@ -1141,10 +1154,7 @@ extern "C" int sdf_features_update_positions(sdf_features f, const float *vertic
     if (!f || !vertices) return SDF_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     SDF_TRY(cudaMemcpyAsync(f->vpos, vertices, sizeof(float) * 3 * f->V, cudaMemcpyDeviceToDevice, s));
-    SDF_TRY(cudaMemsetAsync(f->ctr->cls, 0, sizeof(f->ctr->cls), s));
-    SDF_TRY(cudaMemsetAsync(&f->ctr->status, 0, sizeof(unsigned), s));  // re-evaluated below
-    SDF_TRY(cudaMemsetAsync(f->ctr->prec, 0, sizeof(f->ctr->prec), s));  // precision terms, likewise
-    SDF_TRY(cudaMemsetAsync(f->ctr->box_mom, 0, sizeof(f->ctr->box_mom), s));
+    SDF_TRY(launch_dep(k_positions_init, dim3(1), dim3(32), 0, s, f->ctr));  // re-evaluated below
     return build_records(f, s);
 }
 
