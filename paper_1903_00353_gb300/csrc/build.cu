@@ -166,10 +166,9 @@ __device__ __forceinline__ void run_heads(const uint32_t *vals, const float *sou
 // The mixed runs (grid-stride over the device-side count): re-ordered by (coordinate bits, soup index)
 // so that equal vertices become contiguous, runs of up to WELD_SHORT entries by the thread itself
 // (insertion sort), longer ones are listed for k_weld_sort_runs, one block per run.
-constexpr int WELD_SHORT = 32, WELD_BLOCK_MAX = 2048;
+constexpr int WELD_SHORT = 32, WELD_TILE = 2048;
 __global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *soup, int64_t n, const int32_t *mixed,
-                           const unsigned *n_mixed, uint32_t *head, int2 *long_runs, int64_t long_cap,
-                           unsigned *n_long) {
+                           const unsigned *n_mixed, uint32_t *head, int2 *long_runs, unsigned *n_long) {
     dep_wait();
     dep_next();
     const int64_t nm = *n_mixed;
@@ -177,14 +176,11 @@ __global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *so
         const int64_t i = mixed[r];
         int64_t e = i + 1;
         while (e < n && keys[e] == keys[i]) e++;
-        if (e - i > WELD_SHORT && e - i <= WELD_BLOCK_MAX) {
-            const unsigned slot = atomicAdd(n_long, 1u);
-            if ((int64_t)slot < long_cap) {
-                long_runs[slot] = make_int2((int)i, (int)(e - i));
-                continue;
-            }
+        if (e - i > WELD_SHORT) {  // at most n / (WELD_SHORT + 1) of them: the list holds them all
+            long_runs[atomicAdd(n_long, 1u)] = make_int2((int)i, (int)(e - i));
+            continue;
         }
-        for (int64_t a = i + 1; a < e; a++) {  // short runs (and runs beyond the block sort's size)
+        for (int64_t a = i + 1; a < e; a++) {
             uint32_t v = vals[a];
             int64_t b = a - 1;
             while (b >= i && less_xyz(soup, v, vals[b])) { vals[b + 1] = vals[b]; b--; }
@@ -194,50 +190,94 @@ __global__ void k_weld_fix(const uint64_t *keys, uint32_t *vals, const float *so
     }
 }
 
-// The listed long mixed runs, one block per run (grid-stride over the device-side count): the
-// run's (x, y, z bits, soup index) records are sorted in shared memory by a bitonic network over
-// the next power of two (padding sorts last), then written back.  Any total order of the
-// coordinate bits makes equal vertices contiguous; -0 is read as +0.
-__global__ void __launch_bounds__(256) k_weld_sort_runs(const int2 *long_runs, const unsigned *n_long, int64_t long_cap,
-                                                        uint32_t *vals, const float *soup, uint32_t *head) {
+// Record of a soup corner (x, y, z bits, soup index) and its order, that of less_xyz.  Any total order of
+// the coordinate bits makes equal vertices contiguous; -0 is read as +0.
+__device__ __forceinline__ uint4 weld_rec(const float *soup, uint32_t v) {
+    return make_uint4(__float_as_uint(canon_zero(soup[3 * (int64_t)v])),
+                      __float_as_uint(canon_zero(soup[3 * (int64_t)v + 1])),
+                      __float_as_uint(canon_zero(soup[3 * (int64_t)v + 2])), v);
+}
+__device__ __forceinline__ void order_recs(uint4 *rec, int t, int u) {
+    const uint4 a = rec[t], b = rec[u];
+    if (a.x != b.x ? a.x > b.x : (a.y != b.y ? a.y > b.y : (a.z != b.z ? a.z > b.z : a.w > b.w))) {
+        rec[t] = b;
+        rec[u] = a;
+    }
+}
+__device__ __forceinline__ void order_vals(uint32_t *vals, const float *soup, int64_t t, int64_t u) {
+    const uint32_t a = vals[t], b = vals[u];
+    if (less_xyz(soup, b, a)) {
+        vals[t] = b;
+        vals[u] = a;
+    }
+}
+// pair number t of a merge step: (t, mirror image) within blocks of k, or (t, t + j) within blocks of 2 j
+__device__ __forceinline__ int64_t pair_low(int64_t t, int64_t j) { return 2 * t - (t & (j - 1)); }
+__device__ __forceinline__ int64_t mirror(int64_t t, int64_t k) { return t ^ (k - 1); }
+
+// The listed long mixed runs, one block per run (grid-stride over the device-side count), by a bitonic
+// network whose comparators all put the smaller entry first (each merge starts with a mirrored step), so
+// that a run of any length is sorted as if entries past its end were larger than all.  The steps that
+// stay within WELD_TILE entries run on records in shared memory, a tile at a time; the few steps of a
+// longer run that span tiles gather from the soup.  The build of 722 k triangles in one Morton cell (1024
+// runs of about 2115 entries) takes 2.6 ms; with runs of more than 2048 entries sorted by one thread each,
+// by insertion, it took 1300 ms (the threads, listed side by side, on four SMs).
+__global__ void __launch_bounds__(256) k_weld_sort_runs(const int2 *long_runs, const unsigned *n_long, uint32_t *vals,
+                                                        const float *soup, uint32_t *head) {
     dep_wait();
     dep_next();
-    __shared__ uint4 rec[WELD_BLOCK_MAX];
-    const int64_t nl = min((int64_t)*n_long, long_cap);
+    __shared__ uint4 rec[WELD_TILE];
+    const int64_t nl = *n_long;
     for (int64_t r = blockIdx.x; r < nl; r += gridDim.x) {
         const int2 run = long_runs[r];
-        int m = 1;
-        while (m < run.y) m <<= 1;
-        for (int t = threadIdx.x; t < m; t += blockDim.x) {
-            if (t < run.y) {
-                const uint32_t v = vals[run.x + t];
-                rec[t] = make_uint4(__float_as_uint(canon_zero(soup[3 * (int64_t)v])),
-                                    __float_as_uint(canon_zero(soup[3 * (int64_t)v + 1])),
-                                    __float_as_uint(canon_zero(soup[3 * (int64_t)v + 2])), v);
-            } else {
-                rec[t] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
-            }
-        }
-        __syncthreads();
-        for (int k = 2; k <= m; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int t = threadIdx.x; t < m; t += blockDim.x) {
-                    const int u = t ^ j;
-                    if (u > t) {
-                        const uint4 a = rec[t], b = rec[u];
-                        const bool gt = a.x != b.x ? a.x > b.x : (a.y != b.y ? a.y > b.y : (a.z != b.z ? a.z > b.z : a.w > b.w));
-                        if (gt == ((t & k) == 0)) {  // ascending where t & k == 0
-                            rec[t] = b;
-                            rec[u] = a;
-                        }
+        uint32_t *const rv = vals + run.x;
+        const int64_t len = run.y;
+        int64_t m = 1;  // the run's length rounded up to a power of two
+        while (m < len) m <<= 1;
+        const int mt = (int)(m < WELD_TILE ? m : WELD_TILE);
+        // records of the tile from entry `base` on: merges of 2 .. mt entries (sort), or the last steps of
+        // a longer merge, from distance mt / 2 down
+        auto tile_steps = [&](int64_t base, bool sort) {
+            for (int t = threadIdx.x; t < mt; t += blockDim.x)
+                rec[t] = base + t < len ? weld_rec(soup, rv[base + t])
+                                        : make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+            __syncthreads();
+            for (int k = sort ? 2 : 2 * mt; k <= (sort ? mt : 2 * mt); k <<= 1) {
+                if (sort) {
+                    for (int t = threadIdx.x; t < mt / 2; t += blockDim.x) {
+                        const int a = (int)pair_low(t, k / 2);
+                        order_recs(rec, a, (int)mirror(a, k));
                     }
+                    __syncthreads();
+                }
+                for (int j = k >> 2; j > 0; j >>= 1) {
+                    for (int t = threadIdx.x; t < mt / 2; t += blockDim.x) {
+                        const int a = (int)pair_low(t, j);
+                        order_recs(rec, a, a + j);
+                    }
+                    __syncthreads();
+                }
+            }
+            for (int t = threadIdx.x; t < mt && base + t < len; t += blockDim.x) rv[base + t] = rec[t].w;
+            __syncthreads();
+        };
+        for (int64_t base = 0; base < len; base += mt) tile_steps(base, true);
+        for (int64_t k = 2 * WELD_TILE; k <= m; k <<= 1) {  // merges that span tiles
+            for (int64_t t = threadIdx.x; t < m / 2; t += blockDim.x) {
+                const int64_t a = pair_low(t, k / 2), b = mirror(a, k);
+                if (b < len) order_vals(rv, soup, a, b);
+            }
+            __syncthreads();
+            for (int64_t j = k >> 2; j >= WELD_TILE; j >>= 1) {
+                for (int64_t t = threadIdx.x; t < m / 2; t += blockDim.x) {
+                    const int64_t a = pair_low(t, j);
+                    if (a + j < len) order_vals(rv, soup, a, a + j);
                 }
                 __syncthreads();
             }
+            for (int64_t base = 0; base < len; base += mt) tile_steps(base, false);
         }
-        for (int t = threadIdx.x; t < run.y; t += blockDim.x) vals[run.x + t] = rec[t].w;
-        __syncthreads();
-        run_heads(vals, soup, run.x, run.x + (int64_t)run.y, threadIdx.x, blockDim.x, head);
+        run_heads(vals, soup, run.x, run.x + len, threadIdx.x, blockDim.x, head);
     }
 }
 
@@ -1058,8 +1098,8 @@ extern "C" int sdf_build_features(const float *soup, int64_t n_tri, uint32_t fla
     B_TRY(radix_sort_u64(keys, vals, kalt, valt, n, 40, rtmp, scan_state, s, err));
     B_TRY(launch_dep(k_weld_heads, dim3(nblk(n)), dim3(BT), 0, s, keys, vals, soup, n, valt, mixed, n_mixed));
     B_TRY(launch_dep(k_weld_fix, dim3((unsigned)std::min<int64_t>(nblk(n / 2 + 1), 2 * 152)), dim3(BT), 0, s, keys, vals,
-                     soup, n, mixed, n_mixed, valt, long_runs, long_cap, n_long));
-    B_TRY(launch_dep(k_weld_sort_runs, dim3(2 * 152), dim3(256), 0, s, long_runs, n_long, long_cap, vals, soup, valt));
+                     soup, n, mixed, n_mixed, valt, long_runs, n_long));
+    B_TRY(launch_dep(k_weld_sort_runs, dim3(2 * 152), dim3(256), 0, s, long_runs, n_long, vals, soup, valt));
     // head[i] = number of run heads before i, head[n] = V (so head[i+1] is the inclusive count at i)
     B_TRY(scan_exclusive_u32(valt, head, n, true, scan_state, s, err));
     uint32_t Vh = 0;
