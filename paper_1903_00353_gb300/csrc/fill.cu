@@ -77,15 +77,17 @@ __global__ void __launch_bounds__(256) k_fill_rows(const FillProb *P, const long
         const FillProb pr = P[p];
         float *row = pr.dist + (r - rbase[p]) * (long long)pr.nx;
         int first = 0, carry = 0;
-        for (int s0 = 0; s0 < pr.nx; s0 += 1024) {
-            const int chunks = min(32, (pr.nx - s0 + 31) >> 5);
+        // (unsigned: the ends of steps of 1024 and of eight chunks may lie beyond the largest int)
+        const unsigned nx = (unsigned)pr.nx;
+        for (unsigned s0 = 0; s0 < nx; s0 += 1024) {
+            const int chunks = (int)min(32u, (nx - s0 + 31) >> 5);
             unsigned known = 0, neg = 0;
             for (int c0 = 0; c0 < chunks; c0 += 8) {
                 float v[8];
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
-                    const int x = s0 + (c0 + u) * 32 + lane;
-                    v[u] = x < pr.nx ? row[x] : INFINITY;
+                    const unsigned x = s0 + (c0 + u) * 32 + lane;
+                    v[u] = x < nx ? row[x] : INFINITY;
                 }
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
@@ -102,15 +104,15 @@ __global__ void __launch_bounds__(256) k_fill_rows(const FillProb *P, const long
             if (had == 0 && carry != 0) {  // the first band point of the row: it decides all before it
                 first = __shfl_sync(FULL_MASK, in, 0);
                 if (first < 0)
-                    for (int x = lane; x < s0; x += 32) row[x] = -INFINITY;
+                    for (unsigned x = lane; x < s0; x += 32) row[x] = -INFINITY;
             }
             // the chunks that can hold inside points
             for (unsigned todo = __ballot_sync(FULL_MASK, lane < chunks && (in < 0 || neg != 0)); todo; todo &= todo - 1) {
                 const int c = __ffs(todo) - 1;
                 const unsigned ck = __shfl_sync(FULL_MASK, known, c), cn = __shfl_sync(FULL_MASK, neg, c);
                 const int s = sign_at(ck, cn, __shfl_sync(FULL_MASK, in, c));
-                const int x = s0 + c * 32 + lane;
-                if (x < pr.nx && !((ck >> lane) & 1u) && s < 0) row[x] = -INFINITY;
+                const unsigned x = s0 + c * 32 + lane;
+                if (x < nx && !((ck >> lane) & 1u) && s < 0) row[x] = -INFINITY;
             }
         }
         if (lane == 0) rowsign[r] = (int8_t)first;  // 0: resolved by the line passes
@@ -128,17 +130,17 @@ __global__ void __launch_bounds__(256) k_fill_lines_y(const FillProb *P, const l
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long L = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); L < l_tot; L += warps) {
         const int p = find_row_prob(zbase, n, L);
-        const int len = P[p].ny;
+        const unsigned len = (unsigned)P[p].ny;
         int8_t *e = rowsign + rbase[p] + (L - zbase[p]) * (long long)len;
         int carry = 0;
-        for (int s0 = 0; s0 < len; s0 += 1024) {
-            const int chunks = min(32, (len - s0 + 31) >> 5);
+        for (unsigned s0 = 0; s0 < len; s0 += 1024) {
+            const int chunks = (int)min(32u, (len - s0 + 31) >> 5);
             unsigned known = 0, neg = 0;
             for (int c0 = 0; c0 < chunks; c0 += 8) {
                 int v[8];
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
-                    const int i = s0 + (c0 + u) * 32 + lane;
+                    const unsigned i = s0 + (c0 + u) * 32 + lane;
                     v[u] = i < len ? (int)e[i] : 0;
                 }
 #pragma unroll
@@ -155,12 +157,12 @@ __global__ void __launch_bounds__(256) k_fill_lines_y(const FillProb *P, const l
             if (carry == 0) continue;  // nothing known so far
             if (had == 0) {
                 const int8_t m = (int8_t)(2 * __shfl_sync(FULL_MASK, in, 0));
-                for (int i = lane; i < s0; i += 32) e[i] = m;
+                for (unsigned i = lane; i < s0; i += 32) e[i] = m;
             }
             for (int c = 0; c < chunks; c++) {
                 const unsigned ck = __shfl_sync(FULL_MASK, known, c), cn = __shfl_sync(FULL_MASK, neg, c);
                 const int s = sign_at(ck, cn, __shfl_sync(FULL_MASK, in, c));
-                const int i = s0 + c * 32 + lane;
+                const unsigned i = s0 + c * 32 + lane;
                 if (i < len && !((ck >> lane) & 1u)) e[i] = (int8_t)(2 * s);
             }
         }
