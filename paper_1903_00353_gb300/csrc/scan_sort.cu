@@ -198,6 +198,7 @@ cudaError_t scan_exclusive_u32(const uint32_t *in, uint32_t *out, int64_t n, boo
 // keys) still spread over every SM instead of a few dozen CTAs.
 namespace {
 constexpr int RS_THREADS = 256, RS_WARPS = RS_THREADS / 32, RADIX = 256;
+constexpr int RS_ITEMS_MIN = 2;  // keys per thread of the smallest sorts (rs_items)
 template <int ITEMS>
 constexpr size_t rs_smem() {
     return (size_t)RS_THREADS * ITEMS * (sizeof(uint64_t) + sizeof(uint32_t)) +
@@ -312,13 +313,16 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t *kin, 
 // by other CTAs is read past L1 (ld.global.cg).  Against the three launches per pass above (a
 // histogram, a scan and a scatter) this makes 1 launch per sort.
 //
-// With at most RS_DIRECT tiles step (2) and its barrier are left out: each CTA reads all tiles' counts
-// itself (1 KB per tile, tile-major, sixteen loads in flight) and sums them per digit.  A pass is then
-// bound by two barriers, about 1.5 us each, and the latency of its loads; five passes over 64 tiles (the
-// weld of 10,800 triangles) took 60 us with three barriers, now 42.  For more tiles the counts that
-// every CTA reads grow with the square of their number (147 tiles: 119 us against 63).
+// A sort of fewer than RS_DIRECT keys leaves out step (2) and its barrier: each CTA reads all tiles'
+// counts itself (1 KB per tile, tile-major, sixteen loads in flight) and sums them per digit.  A pass is
+// then bound by two barriers, about 1.5 us each, and the latency of its loads, which grows with the
+// tiles; with three barriers it is bound by those and, below 64 tiles, by the few CTAs that scan the counts.
+// us per sort, direct / three barriers, by tiles of 512 keys:
+//   weld (5 passes)   16: 37 / 107   64: 44 / 60   96: 52 / 58   112: 56 / 58     120: 58 / 58   128: 52 / 55
+//   faces (2 passes)  22: 15 / 36    67: 17 / 25   83: 19 / 24   98: 23.3 / 23.4  114: 26 / 24   127: 23.4 / 24.2
+// so the two meet at about 110 tiles; the line is at 128, up to where a digit's counts fit 16 bits.
 constexpr unsigned RS_POLL_LIMIT = 1u << 20;
-constexpr unsigned RS_DIRECT = 128;
+constexpr int64_t RS_DIRECT = 65536;  // keys: all tiles' count of a digit << 16 | that of the tiles before
 
 // Grid barrier of a cooperative launch on bar[0] (arrivals, 0 between barriers) and bar[1]
 // (generation): the last CTA to arrive clears the arrivals and advances the generation; the others
@@ -380,7 +384,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_one(uint64_t *keys, uint32_t 
     const int cnt = (int)(n - tile0 < (int64_t)TILE ? n - tile0 : (int64_t)TILE);
     const uint32_t lt_mask = (1u << lane) - 1u;
     uint32_t *mycnt = wcnt + warp * RADIX;
-    const bool direct = nb <= RS_DIRECT && n < 65536;
+    // (a sort in larger tiles has at least 152 of them, rs_items: too many keys)
+    const bool direct = ITEMS == RS_ITEMS_MIN && n < RS_DIRECT;
     for (int p = 0; p < passes; p++) {
         const int shift = 8 * p;
         // (1) ranks within the tile: lanes in order within a warp, warps in order (stable)
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_one(uint64_t *keys, uint32_t 
         }
         // (3) global start of the tile's run of digit d: the totals of the smaller digits plus the
         // counts of digit d in the tiles before this one
-        if (direct) {  // four digits per thread, a quarter of the tiles; (all << 16 | before) fits: n < 2^16
+        if (direct) {  // four digits per thread, a quarter of the tiles; all << 16 | before per digit
             uint32_t *part = reinterpret_cast<uint32_t *>(skey);  // [4][RADIX], free until the scatter
             const unsigned dq = threadIdx.x & 63, quarter = threadIdx.x >> 6;
             uint4 sum = make_uint4(0u, 0u, 0u, 0u);
@@ -478,14 +483,14 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_one(uint64_t *keys, uint32_t 
     }
 }
 
-// keys per thread: the largest of 8, 4, 2 that still gives at least one tile per SM (the SM
+// keys per thread: the largest of 8, 4, RS_ITEMS_MIN that still gives at least one tile per SM (the SM
 // count of this part; the count only changes the choice, not the result).  16 keys per thread
 // would need 127 registers, two CTAs per SM: the 6.3 M-key sort of the knot tube ran its scatter
 // passes faster with 8.
 int rs_items(int64_t n) {
-    for (int items = 8; items > 2; items >>= 1)
+    for (int items = 8; items > RS_ITEMS_MIN; items >>= 1)
         if ((n + RS_THREADS * items - 1) / (RS_THREADS * items) >= 152) return items;
-    return 2;
+    return RS_ITEMS_MIN;
 }
 
 template <int ITEMS>
@@ -580,14 +585,14 @@ cudaError_t rs_one(uint64_t *keys, uint32_t *vals, int64_t n, int bits, void *tm
 // histograms of a sort of at most n keys: sized for the smallest tile (the most tiles), so that
 // they also hold those of any shorter sort, whatever tile size that one picks
 size_t radix_tmp_bytes(int64_t n) {
-    const int64_t tile = (int64_t)RS_THREADS * 2;
+    const int64_t tile = (int64_t)RS_THREADS * RS_ITEMS_MIN;
     int64_t nb = (n + tile - 1) / tile;
     return ((size_t)nb * RADIX + RADIX + 64) * sizeof(uint32_t);  // + the one-launch sort's digit totals
 }
 
 // the scan state a sort of at most n keys needs (its digit histograms are scanned)
 size_t radix_scan_state_bytes(int64_t n) {
-    const int64_t tile = (int64_t)RS_THREADS * 2;
+    const int64_t tile = (int64_t)RS_THREADS * RS_ITEMS_MIN;
     return scan_state_bytes(((n + tile - 1) / tile) * RADIX);
 }
 
