@@ -534,10 +534,11 @@ __device__ __forceinline__ float eval_any(const Feat &F, const GridP &g, int typ
 // computed once per (region, tile) and kept in shared memory, lower bounds from the front and
 // upper bounds from the back of the region's slots, so a row costs one FMA pair and a min or max
 // per plane (unused slots hold the neutral upper bound +1e30, so every row runs all KMAX slots
-// without branching).  Vertex regions keep at most MAXVP of their planes: dropping planes only enlarges the
+// without branching).  Vertex regions keep at most VERT_PLANES of their planes: dropping planes only enlarges the
 // region, and a point outside the exact vertex region has a strictly closer point on an incident
 // edge.  Faces have 5 planes, edges 4.
-constexpr int KMAX = 6, MAXVP = 6;
+constexpr int KMAX = 6;
+static_assert(VERT_PLANES <= KMAX, "a region's planes must fit its slots");
 enum { Q_NONE = 0, Q_EDGE = 1, Q_VERT = 2 };  // kinds of quadratic row bound
 
 template <int TY, int TZ, int NT>
@@ -720,7 +721,7 @@ __device__ __forceinline__ int setup_region(const Feat &F, const GridP &g, int2 
         kind = Q_EDGE;
     } else {
         const float4 v = __ldg(F.vert_rec + 3 * id), nv = __ldg(F.vert_rec + 3 * id + 1);
-        const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), MAXVP);
+        const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), VERT_PLANES);
         for (int k = 0; k < cnt; k++) {
             const float4 P = __ldg(F.vert_plane + s0 + k);
             rc.add(along(P, ax), P.w);
@@ -2060,7 +2061,7 @@ __device__ __forceinline__ bool region_contains(const Feat &F, const GridP &g, i
         const float3 u = p - f3(v);
         const float R = g.W + e;
         if (dot3(u, u) > R * R) return false;
-        const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), MAXVP);
+        const int s0 = __float_as_int(v.w), cnt = min(__float_as_int(nv.w), VERT_PLANES);
         for (int k = 0; k < cnt; k++) {
             const float4 P = __ldg(F.vert_plane + s0 + k);
             if (dot3(f3(P), p) + P.w < -e) return false;

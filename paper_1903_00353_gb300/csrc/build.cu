@@ -595,7 +595,6 @@ __device__ __forceinline__ float corner_angle(float3 e1, float3 e2) {
 
 constexpr int VL = 8;      // lanes per vertex in k_vertex_records
 constexpr int VMAXS = 24;  // corners of a fan staged in shared memory (and cone-searched)
-constexpr int NARROW_VP = 6;  // planes of a vertex region that the narrow band tests (MAXVP in band.cu)
 
 __device__ __forceinline__ float gsum8(float v) {
     v += __shfl_xor_sync(0xffffffffu, v, 4, VL);
@@ -776,7 +775,7 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
         // if all its rays lie within 89 degrees of +N_alpha (or of -N_alpha).  The flags and bounds
         // below are uniform over the 8 lanes of a vertex after the group reductions.
         // Two more bounds tell the narrow band which regions hold no grid point (feature_box); the tile
-        // kernel tests a vertex's first NARROW_VP planes, so both are left out for larger fans.
+        // kernel tests a vertex's first VERT_PLANES planes, so both are left out for larger fans.
         //  - No feasible ray: the region is v alone, and {y : y.e_j <= t} lies within t / mu of it, mu the
         //    distance of the hull of the e_j from the origin inside it.  At the nearest facet (a, b, c),
         //    u.e_a = u.e_b = u.e_c = mu with u its normal; some two of them, a and b, are at most 120 degrees
@@ -843,8 +842,8 @@ __global__ void __launch_bounds__(BT, 4) k_vertex_records(const int32_t *vert_st
                 else if (conc_cone) cone = make_float4(-1.f, 0.f, 0.f, cmin - 2e-3f);
                 else if (search && any && all_pos) cone = make_float4(1.f, 0.f, 0.f, cpos - 2e-3f);
                 else if (search && any && all_neg) cone = make_float4(-1.f, 0.f, 0.f, cng - 2e-3f);
-                else if (search && !any && deg <= NARROW_VP && viol > 1e-3f) cone.w = -2.f - 4.f / viol;
-                if (deg <= NARROW_VP && cmin > 0.9f && asum < 9.42f) {
+                else if (search && !any && deg <= VERT_PLANES && viol > 1e-3f) cone.w = -2.f - 4.f / viol;
+                if (deg <= VERT_PLANES && cmin > 0.9f && asum < 9.42f) {
                     const float z = zmax / Nlen * 1.001f + 1e-5f, z2 = fminf(z * z, 0.5f);
                     const float ca = cospif(0.318309886f * amax) - 1e-5f - z2, cg = fmaxf(ca < 0.f ? ca / (1.f - z2) : ca, -1.f);
                     const float width = 0.999f * sqrtf(0.5f * (1.f + cg) * (1.f - z2));

@@ -23,6 +23,11 @@ enum : unsigned {
 // vertex / edge classes (Section 3.1, Section 3.2)
 enum : int8_t { CLS_FLAT = 0, CLS_CONVEX = 1, CLS_CONCAVE = -1, CLS_SADDLE = 2 };
 
+// planes of a vertex region that the narrow band tests: a vertex of more corners keeps a larger region
+// (the row set-up holds this many), and only of smaller ones may the build's bounds tell whether the
+// region holds a grid point
+constexpr int VERT_PLANES = 6;
+
 // tile of the narrow-band kernel: TX x TY x TZ grid points (x fastest)
 constexpr int TILE_X = 32, TILE_Y = 8, TILE_Z = 8;
 constexpr int TILE_PTS = TILE_X * TILE_Y * TILE_Z;
