@@ -1297,7 +1297,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, c
             continue;
         }
         {  // a band tile, or an item of a split tile
-            const bool is_band = true;
             int64_t tile;
             int split_slot = -1, split_i = 0, split_n = 1;
             if (SPLIT) {
@@ -1320,21 +1319,19 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, c
             const int64_t plane = (int64_t)g.nx * g.ny;
             float *dist = pr.dist;
             int32_t *winner = pr.winner;
-            if (is_band) {
-                const uint32_t *st = o.bin_start + 3 * tile;
-                int64_t q0 = min((int64_t)st[0], o.pair_cap), q3 = min((int64_t)st[3], o.pair_cap);
-                if (SPLIT) {  // this item's contiguous part of the tile's pairs
-                    const int64_t np = q3 - q0;
-                    const int64_t qa = q0 + np * split_i / split_n, qb = q0 + np * (split_i + 1) / split_n;
-                    q0 = qa;
-                    q3 = qb;
-                }
-                process_band_tile<TY, TZ, NT>(pr.F, g, o.pairs, q0, q3, x0, y0, z0, S, cand, rows, hits);
-                __syncthreads();  // every merge is in before the decode
-                if (threadIdx.x == 0) pairs += (unsigned)(q3 - q0);
-                if (SPLIT && !split_merge<TP, NT>(o, S.key, split_slot, split_n, s_last)) continue;
+            const uint32_t *st = o.bin_start + 3 * tile;
+            int64_t q0 = min((int64_t)st[0], o.pair_cap), q3 = min((int64_t)st[3], o.pair_cap);
+            if (SPLIT) {  // this item's contiguous part of the tile's pairs
+                const int64_t np = q3 - q0;
+                const int64_t qa = q0 + np * split_i / split_n, qb = q0 + np * (split_i + 1) / split_n;
+                q0 = qa;
+                q3 = qb;
             }
-            const bool list = LIST && is_band && pr.list != nullptr;
+            process_band_tile<TY, TZ, NT>(pr.F, g, o.pairs, q0, q3, x0, y0, z0, S, cand, rows, hits);
+            __syncthreads();  // every merge is in before the decode
+            if (threadIdx.x == 0) pairs += (unsigned)(q3 - q0);
+            if (SPLIT && !split_merge<TP, NT>(o, S.key, split_slot, split_n, s_last)) continue;
+            const bool list = LIST && pr.list != nullptr;
             const bool vec_rows = pr.vec && cx1 == x0 + TILE_X - 1;
             unsigned emask = 0;  // this thread's points that go to the band list (bit: decode order)
             if (vec_rows) {
@@ -1345,19 +1342,17 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, c
                     if (gj > cy1 || gk > cz1) continue;
                     const int x = (threadIdx.x & 7) * 4;
                     const int64_t idx = (int64_t)gk * plane + (int64_t)gj * g.nx + x0 + x;
-                    float4 v = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-                    int4 wv = make_int4(-1, -1, -1, -1);
-                    if (is_band) {
-                        const unsigned long long *kp = S.key + r * TILE_X + x;
-                        bool e0, e1, e2, e3;
-                        v.x = decode_key(kp[0], g, o, idx, p, wv.x, band, overflow, e0);
-                        v.y = decode_key(kp[1], g, o, idx + 1, p, wv.y, band, overflow, e1);
-                        v.z = decode_key(kp[2], g, o, idx + 2, p, wv.z, band, overflow, e2);
-                        v.w = decode_key(kp[3], g, o, idx + 3, p, wv.w, band, overflow, e3);
-                        if (list) {
-                            const int sh = 4 * ((r - (int)(threadIdx.x >> 3)) / (NT / 8));
-                            emask |= ((unsigned)e0 | (unsigned)e1 << 1 | (unsigned)e2 << 2 | (unsigned)e3 << 3) << sh;
-                        }
+                    float4 v;
+                    int4 wv;
+                    const unsigned long long *kp = S.key + r * TILE_X + x;
+                    bool e0, e1, e2, e3;
+                    v.x = decode_key(kp[0], g, o, idx, p, wv.x, band, overflow, e0);
+                    v.y = decode_key(kp[1], g, o, idx + 1, p, wv.y, band, overflow, e1);
+                    v.z = decode_key(kp[2], g, o, idx + 2, p, wv.z, band, overflow, e2);
+                    v.w = decode_key(kp[3], g, o, idx + 3, p, wv.w, band, overflow, e3);
+                    if (list) {
+                        const int sh = 4 * ((r - (int)(threadIdx.x >> 3)) / (NT / 8));
+                        emask |= ((unsigned)e0 | (unsigned)e1 << 1 | (unsigned)e2 << 2 | (unsigned)e3 << 3) << sh;
                     }
                     if (dist) __stcs(reinterpret_cast<float4 *>(dist + idx), v);
                     if (winner) __stcs(reinterpret_cast<int4 *>(winner + idx), wv);
@@ -1370,14 +1365,14 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, c
                     const int64_t idx = (int64_t)gk * plane + (int64_t)gj * g.nx + gi;
                     int wid = -1;
                     bool en = false;
-                    const float val = is_band ? decode_key(S.key[e], g, o, idx, p, wid, band, overflow, en) : INFINITY;
+                    const float val = decode_key(S.key[e], g, o, idx, p, wid, band, overflow, en);
                     if (list && en) emask |= 1u << ((e - (int)threadIdx.x) / NT);
                     if (dist) __stcs(dist + idx, val);
                     if (winner) __stcs(winner + idx, wid);
                 }
             }
             if (list) list_write<TY, TZ, NT>(pr, S, emask, x0, y0, z0, vec_rows, list_ovf);
-            if (is_band) __syncthreads();  // keys are reused by the next band tile
+            __syncthreads();  // keys are reused by the next band tile
         }
     }
     atomicAdd(&s_cand, cand);
