@@ -173,7 +173,7 @@ int sdf_features_update_positions(sdf_features f, const float *vertices, void *s
  * per point the value of smallest magnitude (Algorithm 1) through a packed
  * 64-bit atomicMin of (|d| bits, feature id).  Distances and scan conversion
  * run in FP32; points whose band membership or sign falls inside the FP32
- * error window are re-decided in FP64 from the winner's neighbourhood.
+ * error window are re-decided in FP64 over every region that can hold them.
  *
  *   feats       host array [n] of handles.
  *   grids       host array [n] of grids.

@@ -20,10 +20,10 @@
 //      default; 4x4 and 16x8 for the autotuner) and the (tile, region) pairs, each with the
 //      region's box clipped to the tile, are bucketed per tile and type (count, scan, fill;
 //      a warp's pairs share one atomic per bin); tiles of all problems share one numbering;
-//   2. tile kernel: a persistent grid (6 CTAs of 128 threads per SM, or 4 of 256 on small grids)
+//   2. tile kernel: a persistent grid (6 CTAs of 128 threads per SM, or 4 of 256 in launches over few tiles)
 //      takes work items from two atomic tickets, the band tiles (largest first for batches) and
-//      chunks of the empty tiles.  A band tile keeps the packed keys (|d| bits << 32 | id << 1 | sign) of
-//      its points in shared memory.  One lane per region computes its scan axis and per-plane span
+//      chunks of the empty tiles.  A band tile keeps the packed keys (|d| bits << 32 | id << 2 |
+//      sign uncertain << 1 | negative) of its points in shared memory.  One lane per region computes its scan axis and per-plane span
 //      coefficients (Algorithm 2 restricted to grid lines, with the inclusion tolerance of
 //      Section 10), a warp scan numbers the rows, each lane evaluates one row's span, and the
 //      span points are flattened across lanes, evaluated against the feature and merged with a
@@ -31,8 +31,8 @@
 //      its tile of the dense output (coalesced 16-byte rows), +inf outside the band, optionally
 //      the winners or the compact band list, and queues the few points whose band membership
 //      or sign lies inside the FP32 error window.  Empty tiles are written +inf;
-//   3. patch kernel: re-decides the queued points in FP64 from the winner's neighbourhood (and
-//      appends those it puts in the band to the band list).
+//   3. patch kernel: re-decides the queued points in FP64 over all regions of the point's tile whose box
+//      holds it (and appends those it puts in the band to the band list).
 #include <math.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -208,7 +208,8 @@ __device__ __forceinline__ float cone_reach(float ca, float cth, float sth) {
 // here is one whose row spans are all empty; the others keep their box, since its sides choose the
 // scan axis and so the rounding of the spans.  On the 2.1 M-triangle knot at 512^3 this drops 9 of 10
 // edge and nearly all vertex regions (9.6 to 6.2 M (tile, region) pairs, 43.9 to 29.4 M rows, the tile
-// kernel 896 to 689 us, against 40 us more in the count pass of the binning).  Regions of more than THIN_TOL cells' width or THIN_LEN cells' length hold points anyway and are not tested.
+// kernel 896 to 689 us, against 40 us more in the count pass of the binning).  Regions of more than THIN_TOL
+// cells' half-width or THIN_LEN cells' length mostly hold points and are not tested (the loops stay short).
 constexpr float THIN_LEN = 4.f, THIN_TOL = 0.5f, THIN_REACH = 16.f;  // cells
 constexpr int THIN_GRID = 4096;  // longest grid axis: the index rounding stays below 1/1024 cell
 __device__ __forceinline__ bool thin_holds_point(float3 fa, float3 n, float3 T, float tol, int i0, int i1, int j0,
@@ -1037,11 +1038,13 @@ constexpr int FILL_CHUNK = 32;
 // into a few tiles) is split: while slots last (split_cap), it takes a slot and becomes
 // S = min(ceil(np / SPLIT_PAIRS), SPLIT_MAX_ITEMS) work items, each a contiguous part of its pairs,
 // listed in split_items for the SPLIT launch of the tile kernel; its own entry in band_list becomes
-// -1 (skipped).  An item packs (tile, slot | item << 12 | S << 20).  Many is more than the mean work of
-// a CTA of the launch, within [SPLIT_MIN, SPLIT_MAX]: such a tile would be finished last.  On the
+// -1 (skipped).  An item packs (tile, slot | item << 12 | S << 20).  Many is more than the pairs of the
+// launch by n_ctas, within [SPLIT_MIN, SPLIT_MAX]: such a tile would be finished last.  On the
 // batch of 24 uneven meshes that took the two launches from 69 + 345 us (with 8192 always) to
-// 79 + 283; the knot tube at 512^3, whose tiles of up to 6,000 pairs are no more than a CTA's mean work,
-// loses 90 us when they are split (the items' launch comes first) and keeps them whole.
+// 79 + 283; the knot tube at 512^3, whose tiles of up to 6,000 pairs stay below the line, loses 90 us when they
+// are split (the items' launch comes first).  n_ctas is four per SM whatever the size of the CTAs, a tuned
+// divisor: six per SM, the number that runs in large launches, lets the line sit lower and takes the
+// batch's call from 517 to 545 us, the knot's from 1020 to 1004 at 512^3 and from 1910 to 1890 at 1024^3.
 constexpr int SPLIT_MIN = 2048, SPLIT_MAX = 8192, SPLIT_PAIRS = 1024, SPLIT_MAX_ITEMS = 64, SPLIT_SLOTS = 256;
 // the launch clears tile_hist, tile_cursor, n_split and n_split_items with one memset
 static_assert(offsetof(DevCounters, n_split_items) == offsetof(DevCounters, tile_hist) + 33 * sizeof(unsigned),
@@ -1267,8 +1270,9 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 6) k_tile(const Prob *P, c
             // The CTAs of every fifth SM start on the fill queue, the others on the band tiles.  An
             // SM that writes +inf at full rate slows the band work of its other CTAs nearly as much
             // as the fill is worth, so the fill goes to a few SMs, which take band tiles once it
-            // is done (measured on the 2.1 M-triangle knot at 1024^3: 1.91 ms against 2.01 ms with
-            // half of the CTAs of every SM filling, and 1.37 ms for the band work alone).
+            // is done.  On the 2.1 M-triangle knot at 1024^3 the kernel takes 1.43 ms so, 1.46 with every
+            // seventh SM filling and 1.48 with every tenth (an earlier form of it took 1.91 ms so and
+            // 2.01 with half of the CTAs of every SM filling).
             unsigned smid;
             asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
             const bool filler = smid % 5 == 0;
@@ -1528,7 +1532,7 @@ __device__ __forceinline__ Cand64 vert_cand64(const Feat &F, double3 p, int v) {
 //
 // What bounds it: the latency of the pair and record loads, and the FP64 pipe, which takes some 16
 // cycles per warp instruction whatever the number of active lanes.  So each phase of a round (up to
-// 32 points per block) fills its lanes:
+// PB_PTS points per block) fills its lanes:
 //   0. one thread per point finds the point's tile and pairs;
 //   1. a warp per point reads the tile's pairs, the next four loads in flight, and queues those whose box
 //      holds the point; the distances of 32 queued regions are evaluated at once (a box test per
@@ -2695,7 +2699,11 @@ static Scratch plan_scratch(const Plan &pl) {
 // kernel takes 1.43 ms at 1024^3 (1.57 with 256 threads), a torus forward at 512^3 268 us (283).  On a
 // small grid, where the CTAs get few tiles each, a tile's own time counts and 256 threads are faster:
 // 77 us for a fine box at 64^3 (88 with 128), a fine torus 181 us at 128^3 (235) and 260 us at 256^3
-// (302).  The two meet at about 320^3, 16,000 tiles.
+// (302).  The two meet at about 320^3, 16,000 tiles, for an object that fills the grid.  The line counts all
+// tiles, since how many are band tiles is known on the device only, so a small object in a large grid gets
+// 128: a fine torus over a fifth of a 512^3 grid takes 351 us where 256 would take 302, at a tenth of it
+// 384 (348), while a coarse sphere takes 260 (291), and on 1024^3 both are within 2 % (a coarse sphere
+// 1116, with 256 threads 1263).
 constexpr int64_t SMALL_TILES = 16384;
 
 // the tile kernel: the items of split tiles, then the band tiles and the fill

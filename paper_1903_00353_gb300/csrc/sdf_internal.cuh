@@ -135,7 +135,9 @@ struct sdf_features_s {
     float4 *face_rec = nullptr;     // [T][4] (n, c0) and three inward side planes (m, c)
     float4 *face_box = nullptr;     // [T][2] vertex bounding box lo, hi
     float4 *edge_rec = nullptr;     // [E][5] (a, L) (t, t.a) (-m1, m1.a) (-m2, m2.a) (n1+n2, |n1+n2|)
-    float4 *vert_rec = nullptr;     // [V][3] (v, start) (unit N_alpha, count) (cone axis, cos theta)
+    float4 *vert_rec = nullptr;     // [V][3] (v, start) (unit N_alpha, count) (sign s of the region cone's
+                                    // axis s N_alpha, needle slope, 1 / needle width or 0, cos of the
+                                    // cone's half-angle, -2 for none, or -(2 + 1 / mu): see k_vertex_records
     float4 *vert_plane = nullptr;   // [3T] (-e_j, e_j.v) per incident edge, CSR by vert_start
     int8_t *edge_class = nullptr;   // [E]
     int8_t *vert_class = nullptr;   // [V]
@@ -205,8 +207,8 @@ size_t scan_state_bytes(int64_t n);
 cudaError_t scan_exclusive_u32(const uint32_t *in, uint32_t *out, int64_t n, bool write_total, void *state,
                                cudaStream_t s, unsigned *err);
 // Stable LSD radix sort of (keys, vals) on bits [0, bits).  Buffers *_alt are ping-pong
-// scratch of the same size; the result ends in keys/vals, which may have changed places with them.  tmp holds radix_tmp_bytes(n) bytes of
-// histograms; scan_state is a scan state (as above) of radix_scan_state_bytes(n) bytes.  A sort
+// scratch of the same size; the result ends in keys/vals, which may have changed places with them.
+// tmp holds radix_tmp_bytes(n) bytes of histograms; scan_state is a scan state (as above) of radix_scan_state_bytes(n) bytes.  A sort
 // whose tiles fit on the device at once is one cooperative launch (its grid barrier uses words 2
 // and 3 of the scan state, which every completed sort leaves ready); a barrier wait that runs out
 // sets ST_TIMEOUT in *err.  Otherwise three launches per 8-bit pass.
