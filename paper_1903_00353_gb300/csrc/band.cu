@@ -378,16 +378,20 @@ __device__ __forceinline__ int feat_local(const Feat &F, int fid, int type) {
 // (BIN_COUNT) and the fill pass walk the same pairs; the fill pass takes each bin's slots by
 // counting its count back down to 0 (so the counts need no clearing in between, and end cleared).
 // The count pass leaves the features' boxes in `boxes` (12 bytes a feature), where the fill pass reads
-// them instead of the records (48 to 96 bytes) and the arithmetic; without the array (a grid of more
-// than 65536 points along an axis, the allocation-free entry point) BIN_FILL_AGAIN works them out again.
-enum { BIN_COUNT = 0, BIN_FILL = 1, BIN_FILL_AGAIN = 2 };
+// them instead of the records (48 to 96 bytes) and the arithmetic.  Without the array (a grid of more
+// than 65536 points along an axis, the allocation-free entry point) both passes work them out, and the
+// two must agree to the last bit: a pair that only one of them finds leaves a slot of its bin unwritten
+// or takes one too many.  Compiled apart they do not (the compiler chooses which products of a sum it
+// fuses, and a region next to a grid point is then kept by one pass and dropped by the other), so they are
+// one kernel, BIN_BOTH, told at run time which pass it is.
+enum { BIN_COUNT = 0, BIN_FILL = 1, BIN_BOTH = 2 };
 template <int MODE, int TY, int TZ>
 __global__ void k_bin(const Prob *P, const long long *feat_base, const long long *tile_base, int n, long long f_tot,
                       uint32_t *cnt, const uint32_t *start, int2 *pairs, int64_t pair_cap, DevCounters *ctr,
-                      uint32_t *boxes) {
+                      uint32_t *boxes, int second) {
     dep_wait();
     dep_next();
-    constexpr bool FILL = MODE != BIN_COUNT;
+    const bool fill = MODE == BIN_FILL || (MODE == BIN_BOTH && second);
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     int p = 0, type = 0, fid = 0, ntile = 0;
@@ -412,7 +416,7 @@ __global__ void k_bin(const Prob *P, const long long *feat_base, const long long
             else ok = feature_box<VERT>(F, g, id, i0, i1, j0, j1, k0, k1);
         }
         fid = (int)lid;  // face f -> f, edge e -> T + e, vertex v -> T + E + v (within its problem)
-        if (MODE == BIN_COUNT && boxes) {
+        if (MODE == BIN_COUNT) {
             boxes[gid] = ok ? (uint32_t)i0 | (uint32_t)i1 << 16 : 1u;  // (1, 0): no box
             boxes[f_tot + gid] = (uint32_t)j0 | (uint32_t)j1 << 16;
             boxes[2 * f_tot + gid] = (uint32_t)k0 | (uint32_t)k1 << 16;
@@ -449,10 +453,10 @@ __global__ void k_bin(const Prob *P, const long long *feat_base, const long long
         unsigned base = 0;
         if (has && lane == leader) {
             const unsigned k = (unsigned)__popc(peers);
-            base = FILL ? atomicSub(cnt + bin, k) - k : atomicAdd(cnt + bin, k);
+            base = fill ? atomicSub(cnt + bin, k) - k : atomicAdd(cnt + bin, k);
         }
         base = __shfl_sync(FULL, base, leader);
-        if (FILL && has) {
+        if (fill && has) {
             const int64_t pos = (int64_t)start[bin] + base + __popc(peers & lt_mask);
             if (pos < pair_cap) pairs[pos] = make_int2(ofid, pack_box<TY, TZ>(oi0, oi1, oj0, oj1, ok0, ok1, tx, ty, tz));
             else atomicOr(&ctr->nb_status, ST_PAIR_OVERFLOW);
@@ -2738,11 +2742,13 @@ static int launch_shape(int n, long long f_tot, int64_t n_tiles, const Scratch &
         SDF_TRY(launch_dep(k_front, dim3(blocks), dim3(256), 0, s, const_cast<Prob *>(sc.probs), n, sc.cnt, n_bins,
                            sc.ctr, sc.ticket, sc.split_items ? 3 : 2));
     }
-    SDF_TRY(launch_dep(k_bin<BIN_COUNT, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
-                       f_tot, sc.cnt, (const uint32_t *)nullptr, (int2 *)nullptr, (int64_t)0, sc.ctr, sc.boxes));
+    SDF_TRY(launch_dep(sc.boxes ? k_bin<BIN_COUNT, TY, TZ> : k_bin<BIN_BOTH, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256),
+                       0, s, sc.probs, sc.fbase, sc.tbase, n, f_tot, sc.cnt, (const uint32_t *)nullptr, (int2 *)nullptr,
+                       (int64_t)0, sc.ctr, sc.boxes, 0));
     SDF_TRY(scan_exclusive_u32(sc.cnt, sc.start, n_bins, true, sc.scan_tmp, s, &sc.ctr->nb_status));
-    SDF_TRY(launch_dep(sc.boxes ? k_bin<BIN_FILL, TY, TZ> : k_bin<BIN_FILL_AGAIN, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256), 0, s, sc.probs, sc.fbase, sc.tbase, n,
-                       f_tot, sc.cnt, (const uint32_t *)sc.start, sc.pairs, sc.pair_cap, sc.ctr, sc.boxes));
+    SDF_TRY(launch_dep(sc.boxes ? k_bin<BIN_FILL, TY, TZ> : k_bin<BIN_BOTH, TY, TZ>, dim3(nblk(f_tot, 256)), dim3(256),
+                       0, s, sc.probs, sc.fbase, sc.tbase, n, f_tot, sc.cnt, (const uint32_t *)sc.start, sc.pairs,
+                       sc.pair_cap, sc.ctr, sc.boxes, 1));
     // band / empty tile lists for the persistent tile kernel
     const int lpt = n > 1;  // largest-first order of the band tiles for batches
     const int split_cap = sc.split_items ? SPLIT_SLOTS : 0;
